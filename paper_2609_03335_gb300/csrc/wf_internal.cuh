@@ -111,7 +111,7 @@ struct wf_ctx {
     int rb_pair;                // the pair whose count the pending read-back copies
     void *search_scratch;       // local search: the union's results [max_P], top-k ids, slot pairs
     void *construct_scratch;    // plan constructor: per-plan state of the plans built at once, allocated by its first call
-    int64_t construct_threads;  // plans built at once (a warp each)
+    int64_t construct_threads;  // plans built at once
     int32_t *h_ovf;             // pinned host copy of ovf_count[0]
     cudaEvent_t sweep_done;     // recorded on the caller's stream after the sweeps
     cudaEvent_t ovf_event;      // recorded on side after the read-back
@@ -165,6 +165,8 @@ struct wf_sweep_cfg {
 wf_sweep_cfg wf_sweep_config(const wf_dev_problem &dp);
 int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st);
 size_t wf_stoch_smem(const wf_dev_problem &dp);
+// The status pass (place false: the sweep's producers check the placement).
+int wf_launch_status(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st, bool place);
 size_t wf_batch_smem(const wf_dev_problem &dp);
 int wf_launch_batch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, size_t smem, int32_t *ovf_list,
                     int32_t *ovf_count, cudaStream_t st);

@@ -67,3 +67,13 @@ def test_named_workloads(name, P):
     got, res = build(prob, P, seed=5, jitter=200000, plan_base=3)
     want, ends = oracle.construct(prob, P, seed=5, jitter=200000, plan_base=3)
     check(prob, got, res, want, ends)
+
+
+@pytest.mark.parametrize("D,M,P", [(1, 1, 1), (8, 8, 37), (8, 9, 5), (9, 16, 37), (16, 8, 3), (17, 8, 9), (32, 16, 5)])
+def test_lanes_per_plan(D, M, P):
+    """8, 16 and 32 lanes per plan, both queue words, and warps whose plans are not all there."""
+    rng = np.random.default_rng(100 * D + M)
+    prob = random_problem(rng, n_sessions=9, D=D, M=M)
+    got, res = build(prob, P, seed=3, jitter=5000, plan_base=11)
+    want, ends = oracle.construct(prob, P, seed=3, jitter=5000, plan_base=11)
+    check(prob, got, res, want, ends)
