@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "wf_internal.cuh"
+#include "wf_play.cuh"
 
 namespace {
 
@@ -54,7 +54,6 @@ struct Row {
     int32_t *used;    // [D] resident weights
     int32_t *nres;    // [D] resident model count
     int32_t *stamp;   // [D][M] last dispatch position + 1 using the model, 0 = not resident
-    int32_t *loaded;  // [D] bit m: model m was ever resident on the device (Eq. 12 window terms)
     // With a replica batch limit B = dp.batch (only then laid out):
     int64_t *slot_end;  // [D][B] when each slot of the device's current replica frees
     int64_t *slot_kv;   // [D][B] KV need of the unit in each slot
@@ -76,7 +75,7 @@ __device__ __forceinline__ Row row_at(const wf_dev_problem &dp, uint8_t *base)
     r.used = (int32_t *)(base + o); o += up8(4 * (size_t)dp.D);
     r.nres = (int32_t *)(base + o); o += up8(4 * (size_t)dp.D);
     r.stamp = (int32_t *)(base + o); o += up8(4 * (size_t)dp.D * dp.M);
-    r.loaded = (int32_t *)(base + o); o += up8(4 * (size_t)dp.D);
+    o += up8(4 * (size_t)dp.D);  // (spare: the row's size is part of the static entry point's contract)
     if (dp.batch > 0) {
         r.slot_end = (int64_t *)(base + o); o += 8 * (size_t)dp.D * dp.batch;
         r.slot_kv = (int64_t *)(base + o); o += 8 * (size_t)dp.D * dp.batch;
@@ -123,14 +122,12 @@ __device__ __forceinline__ uint64_t splitmix(uint64_t x)
     return x ^ (x >> 31);
 }
 
-// Run time of activation n on device d; for a latency sample, scaled by the
+// Run time of activation n on device d in a latency sample: scaled by the
 // multiplier drawn from (plan, sample, n) through the integer Box-Muller
 // tables (an arithmetic right shift of the signed product is the floor).
-template <bool kStoch>
 __device__ __forceinline__ int64_t run_time(const wf_dev_problem &dp, int32_t n, int32_t d, uint64_t key)
 {
     const int64_t base = dp.lat[(int64_t)n * dp.D + d];
-    if (!kStoch) return base;
     const uint64_t h = splitmix(key ^ (uint64_t)n);
     const int64_t r = dp.bm_r[h & (uint64_t)(dp.bm_rn - 1)];
     const int64_t c = dp.bm_c[(h >> 32) & (uint64_t)(dp.bm_cn - 1)];
@@ -139,21 +136,15 @@ __device__ __forceinline__ int64_t run_time(const wf_dev_problem &dp, int32_t n,
     return (base * mult + 32768) >> 16;
 }
 
-// One play of a valid plan.  Returns makespan and GPU time; per-session
-// completion latencies are left in row.comp.  With phi, also the window
-// terms of Eq. 12: phi[0] the timely prefetches (a prefetched load that
-// starts before the unit's release and ends by it), phi[1] the lifecycle
-// overhead (the delay each load adds to its unit's start, plus the load time
-// of every reload of a model the device held before).
-template <bool kStoch>
+// One play of a valid plan for one latency sample by one thread.  Returns
+// makespan and GPU time; per-session completion latencies are left in
+// row.comp.
 __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uint64_t key,
-                     int64_t *makespan, int64_t *gpu_total, int64_t *phi = nullptr)
+                     int64_t *makespan, int64_t *gpu_total)
 {
     const int32_t N = dp.N, D = dp.D, M = dp.M, W = dp.W;
-    int64_t timely = 0, life = 0;
     for (int32_t d = 0; d < D; ++d) {
         row.tfree[d] = 0; row.occ[d] = kNone; row.gpu[d] = 0; row.used[d] = 0; row.nres[d] = 0;
-        row.loaded[d] = 0;
     }
     for (int32_t k = 0; k < D * M; ++k) row.stamp[k] = 0;
     for (int32_t w = 0; w < W; ++w) row.comp[w] = kNone;
@@ -177,10 +168,10 @@ __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uin
         const int32_t wm = dp.weight[m];
         int32_t tail = h;
         int64_t kv = dp.peak[(int64_t)h * D + d] - wm;
-        int64_t run = run_time<kStoch>(dp, h, d, key);
+        int64_t run = run_time(dp, h, d, key);
         for (int32_t s = dp.fnext[h]; s >= 0 && bit_at(pr.fuse, s) && pr.place[s] == d; s = dp.fnext[s]) {
             kv = max(kv, (int64_t)dp.peak[(int64_t)s * D + d] - wm);
-            run += run_time<kStoch>(dp, s, d, key);
+            run += run_time(dp, s, d, key);
             tail = s;
         }
 
@@ -202,20 +193,13 @@ __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uin
         if (hit) {
             start = max(tf, rel);
         } else {
-            const bool pf = bit_at(pr.prefetch, h);
-            const int64_t ls = max(tf, pf ? arr : rel);
+            const int64_t ls = max(tf, bit_at(pr.prefetch, h) ? arr : rel);
             if (row.occ[d] == kNone) row.occ[d] = ls;
             row.used[d] += wm;
             row.nres[d] += 1;
             const int64_t le = ls + dp.load[m * D + d];
             start = max(le, rel);
-            if (phi) {
-                timely += pf && ls < rel && le <= rel;
-                if ((row.loaded[d] >> m) & 1) life += dp.load[m * D + d];
-                row.loaded[d] |= 1 << m;
-            }
         }
-        if (phi) life += start - max(tf, rel);
         const int64_t c = start + dp.grant + run;
         row.ctail[tail] = c;
         row.tfree[d] = c;
@@ -240,7 +224,6 @@ __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uin
     for (int32_t w = 0; w < W; ++w) row.comp[w] -= dp.arrival[w];
     *makespan = end - dp.first_arrival;
     *gpu_total = g;
-    if (phi) { phi[0] = timely; phi[1] = life; }
 }
 
 // One play with the replica batch limit B_q (Eq. 11 over every active unit,
@@ -251,9 +234,9 @@ __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uin
 // once resident weights + the KV of the units still running + its own KV
 // fit (idle least-recently-used models are reclaimed first; if that is not
 // enough the unit waits for the next running unit to end).  A unit of
-// another model waits for the device to drain and then hits or loads as in
-// play<false>; its other slots free when the model is ready.  B = 1 gives
-// play<false>'s results.  Deterministic times; retain rows only with B = 1.
+// another model waits for the device to drain and then hits or loads as
+// without the limit; its other slots free when the model is ready.  B = 1
+// gives the results without it.  Deterministic times; retain rows only with B = 1.
 __device__ void play_batched(const wf_dev_problem &dp, const PlanRows &pr, Row &row, int64_t *makespan,
                              int64_t *gpu_total)
 {
@@ -399,58 +382,305 @@ __device__ int64_t select_rank(int64_t *v, int32_t n, int32_t r)
 
 __device__ __forceinline__ int32_t p95_rank(int64_t n) { return (int32_t)((95 * n + 99) / 100 - 1); }
 
-__global__ void __launch_bounds__(kEvalThreads)
-eval_det_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
-                int64_t rows)
+// ---------------------------------------------------------------------------
+// A deterministic plan by one warp.  32 dispatch positions at a time:
+//   A  lane = position: the unit that starts there (Eq. 3-4 chain, its
+//      predecessors, session and arrival), all gathers of a chunk in flight
+//      together;
+//   B  lane = device: residency of the chunk's units in dispatch order
+//      (Eq. 11), the device's queue, weights and count in registers -- the
+//      devices' units are settled side by side;
+//   C  the units one after the other, each by its own position's lane, whose
+//      registers hold the record: releases, loads, starts and finishes (Eq.
+//      2, 5, 7, 10) through finish times and device free times in shared
+//      memory.
+// Step C is the serial chain that bounds a plan; the SM hides it behind the
+// other plans' warps.  Times are TT: u64 on the int64 path; the static entry
+// point plays u32 first, with half the memory and a third of the instructions
+// per maximum, and again on u64 only the plans that leave 32 bits.  1,900
+// plans of N = 2,000 in wf_eval_plans_static: 14.3 ms with a thread per plan
+// and its state in global memory, 0.81 ms with a warp per plan on 64-bit
+// times (108 warp instructions per plan-position), 0.57 ms on u32 times (80).
+// ---------------------------------------------------------------------------
+
+// The warp's working memory: B's answers for C [32], device free times [D],
+// finish times of unit tails [N] and one more entry that stays 0 (the
+// predecessor of a node without one), and the sessions' last finishes plus
+// one [W] (0 = none yet).
+template <typename TT>
+struct WarpMem {
+    uint2 *res;
+    TT *tfree, *ctail, *comp;
+};
+
+__host__ __device__ inline size_t warp_small_bytes(int32_t D) { return 32 * sizeof(uint2) + 8 * (size_t)D; }
+template <typename TT>
+__host__ __device__ inline size_t warp_full_bytes(const wf_dev_problem &dp)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows) return;
-    Row row = row_at(dp, scratch + (size_t)t * row_bytes);
-    for (int64_t p = t; p < pl.P; p += rows) {
-        const PlanRows pr = plan_rows(pl, p);
-        const uint32_t st = plan_status(dp, pr, row);
-        out.status[p] = st;
-        if (st) {
-            out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
-            if (dp.phi_life) dp.phi_timely[p] = dp.phi_life[p] = WF_INF64;
-            continue;
+    return warp_small_bytes(dp.D) + sizeof(TT) * ((size_t)dp.N + 1 + (size_t)dp.W);
+}
+
+// big: the finish and session times, behind the small part in shared memory
+// or in a row of global scratch.
+template <typename TT>
+__device__ __forceinline__ WarpMem<TT> warp_mem(const wf_dev_problem &dp, uint8_t *sm, uint8_t *big)
+{
+    WarpMem<TT> w;
+    w.res = (uint2 *)sm;
+    w.tfree = (TT *)(sm + 32 * sizeof(uint2));
+    w.ctail = (TT *)big;
+    w.comp = w.ctail + dp.N + 1;
+    return w;
+}
+
+// Status bits (Eq. 8-10) by a warp, as plan_status; pos: u16 [N].
+__device__ uint32_t warp_status(const wf_dev_problem &dp, const PlanRows &pr, uint16_t *pos)
+{
+    const int lane = threadIdx.x & 31;
+    const int32_t N = dp.N, D = dp.D;
+    uint32_t st = 0;
+#pragma unroll 4
+    for (int32_t n = lane; n < N; n += 32) {
+        const int32_t d = __ldg(pr.place + n);
+        if (d >= D) st |= WF_ST_DEVICE;
+        else if (__ldg(dp.peak + (int64_t)n * D + d) > __ldg(dp.cap + d)) st |= WF_ST_CAPACITY;
+    }
+#pragma unroll 4
+    for (int32_t i = lane; i < N; i += 32) {
+        const int32_t h = __ldg(pr.order + i);
+        if (h < N) pos[h] = (uint16_t)i;
+        else st |= WF_ST_PERMUTATION;
+    }
+    __syncwarp();
+    // A repeated node leaves some position with another position's entry.
+#pragma unroll 4
+    for (int32_t i = lane; i < N; i += 32) {
+        const int32_t h = __ldg(pr.order + i);
+        if (h < N && pos[h] != (uint16_t)i) st |= WF_ST_PERMUTATION;
+    }
+    st = __reduce_or_sync(0xFFFFFFFFu, st);
+    if (!(st & WF_ST_PERMUTATION)) {
+#pragma unroll 4
+        for (int32_t v = lane; v < N; v += 32) {
+            const uint16_t pv = pos[v];
+            const int32_t e1 = __ldg(dp.pred_off + v + 1);
+            for (int32_t e = __ldg(dp.pred_off + v); e < e1; ++e)
+                if (pos[__ldg(dp.pred_idx + e)] > pv) st |= WF_ST_TOPOLOGY;
         }
-        int64_t mk, g, phi[2];
-        if (dp.batch > 0) play_batched(dp, pr, row, &mk, &g);
-        else play<false>(dp, pr, row, 0, &mk, &g, dp.phi_life ? phi : nullptr);
-        out.makespan_us[p] = mk;
-        out.gpu_us[p] = g;
-        out.p95_us[p] = select_rank(row.comp, dp.W, p95_rank(dp.W));
-        if (dp.phi_life) { dp.phi_timely[p] = phi[0]; dp.phi_life[p] = phi[1]; }
+        st = __reduce_or_sync(0xFFFFFFFFu, st);
+    }
+    __syncwarp();  // pos shares memory with the finish times
+    return st;
+}
+
+// The sessions' completion latencies as ordered unsigned values (sign bit
+// flipped), for warp_select.
+template <typename TT>
+struct LatencyArr {
+    const TT *comp;
+    const int64_t *arrival;
+    __device__ __forceinline__ uint64_t get(int32_t w) const
+    {
+        const uint64_t c = comp[w];
+        return ((c ? c - 1 : (uint64_t)kNone) - (uint64_t)__ldg(arrival + w)) ^ (1ull << 63);
+    }
+};
+
+__device__ __forceinline__ int64_t warp_sum(int64_t v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ int64_t warp_max(int64_t v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
+struct PlayResult {
+    int64_t mk, p95, gpu, timely, life;
+};
+
+// One play of a valid plan; every lane returns the results (mk still counts
+// from 0, not from the first arrival).  kPhi adds the window terms of Eq. 12;
+// Q is the residency queue's word.  With u32 times, false when some time
+// leaves 32 bits (the results are then void).
+template <typename TT, typename Q, bool kPhi>
+__device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const WarpMem<TT> &wm, PlayResult &r)
+{
+    constexpr bool kNarrow = sizeof(TT) == 4;
+    const int lane = threadIdx.x & 31;
+    const int32_t N = dp.N, D = dp.D, W = dp.W;
+    for (int32_t w = lane; w < W; w += 32) wm.comp[w] = 0;
+    for (int32_t d = lane; d < D; d += 32) wm.tfree[d] = 0;
+    if (lane == 0) wm.ctail[N] = 0;
+    // The lane's device: queue, resident count and weights, models ever held.
+    Q queue = 0;
+    uint32_t nres = 0, used = 0, ever = 0;
+    const uint32_t capd = lane < D ? (uint32_t)__ldg(dp.cap + lane) : 0u;
+    TT end = 0;
+    int64_t gsum = 0, timely = 0, life = 0;
+    bool ovf = false;
+    __syncwarp();
+    for (int32_t c0 = 0; c0 < N; c0 += 32) {
+        // A: the unit that starts at this lane's position.
+        const bool in = c0 + lane < N;
+        const int32_t h = in ? __ldg(pr.order + c0 + lane) : 0;
+        const int32_t d = __ldg(pr.place + h);
+        const int32_t fp = __ldg(dp.fprev + h), fn = __ldg(dp.fnext + h);
+        const int32_t m = __ldg(dp.model + h), w = __ldg(dp.session + h);
+        const int32_t e0 = __ldg(dp.pred_off + h), np = __ldg(dp.pred_off + h + 1) - e0;
+        const bool fused = bit_at(pr.fuse, h), pf = bit_at(pr.prefetch, h);
+        const bool unit = in && !(fp >= 0 && fused && __ldg(pr.place + fp) == d);
+        const int64_t arr64 = __ldg(dp.arrival + w);
+        const int32_t wgt = __ldg(dp.weight + m);
+        const int32_t p0 = np > 0 ? __ldg(dp.pred_idx + e0) : N, p1 = np > 1 ? __ldg(dp.pred_idx + e0 + 1) : N;
+        int64_t run64 = (int64_t)dp.grant + __ldg(dp.lat + (int64_t)h * D + d);
+        int32_t kv = __ldg(dp.peak + (int64_t)h * D + d) - wgt, tail = h;
+        if (unit)
+            for (int32_t s = fn; s >= 0 && bit_at(pr.fuse, s) && __ldg(pr.place + s) == d; s = __ldg(dp.fnext + s)) {
+                run64 += __ldg(dp.lat + (int64_t)s * D + d);
+                kv = max(kv, __ldg(dp.peak + (int64_t)s * D + d) - wgt);
+                tail = s;
+            }
+        const TT arr = (TT)arr64, run = (TT)run64;
+        if (kNarrow) ovf |= unit && ((arr64 | run64) >> 32) != 0;
+        const bool drop = unit && pr.retain && !bit_at(pr.retain, tail);
+        const uint32_t w3 = (uint32_t)d | ((uint32_t)m << 5) | (pf ? kPrefetch : 0u) | (drop ? kDrop : 0u);
+        // B: residency of the chunk's units on the lane's device.
+        uint32_t mine = 0;
+        for (int32_t dd = 0; dd < D; ++dd) {
+            const uint32_t on = __ballot_sync(0xFFFFFFFFu, unit && d == dd);
+            if (lane == dd) mine = on;
+        }
+        while (__any_sync(0xFFFFFFFFu, mine)) {
+            const int k = mine ? __ffs((int)mine) - 1 : 0;
+            const uint32_t r1 = __shfl_sync(0xFFFFFFFFu, (uint32_t)kv, k), r3 = __shfl_sync(0xFFFFFFFFu, w3, k);
+            if (mine) {
+                bool missed;
+                uint2 x = settle_lru<Q>(queue, nres, used, capd, r1, r3, dp.weight, dp.load, D, dp.err, missed);
+                if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
+                    const uint32_t mk = (r3 >> 5) & 15u;
+                    x.x |= ((ever >> mk) & 1u) << 31;
+                    ever |= 1u << mk;
+                }
+                wm.res[k] = x;
+                mine &= mine - 1;
+            }
+        }
+        __syncwarp();
+        // C: the units in turn, each by its own lane.
+        const uint2 x = wm.res[lane];
+        const TT ld = kPhi ? x.x & 0x7FFFFFFFu : x.x;
+        const int turn = unit ? lane : 32;
+#pragma unroll 4
+        for (int k = 0; k < 32; ++k) {
+            if (turn == k) {
+                const TT tf = wm.tfree[d];
+                TT rel = max(arr, max(wm.ctail[p0], wm.ctail[p1]));  // Eq. 2, Eq. 7
+                for (int32_t e = 2; e < np; ++e) rel = max(rel, wm.ctail[__ldg(dp.pred_idx + e0 + e)]);
+                // (on a hit the load time is 0 and the prefetch bit cleared)
+                const TT ls = max(tf, (x.y & kPrefetch) ? arr : rel), le = ls + ld;
+                const TT start = max(le, rel), c = start + run;
+                if (kNarrow) ovf |= le < ls || c < start;
+                wm.ctail[tail] = c;
+                wm.tfree[d] = c;
+                wm.comp[w] = max(wm.comp[w], c + 1);
+                end = max(end, c);
+                if (x.y & (kWasEmpty | kEmptied)) {
+                    if (x.y & kWasEmpty) gsum -= (int64_t)ls;
+                    if (x.y & kEmptied) gsum += (int64_t)c;
+                }
+                if (kPhi) {
+                    timely += (x.y & kPrefetch) && ls < rel && le <= rel;
+                    life += (int64_t)(start - max(tf, rel) + (x.x >> 31 ? ld : 0));
+                }
+            }
+            __syncwarp();
+        }
+        if (kNarrow && __any_sync(0xFFFFFFFFu, ovf)) return false;
+    }
+    const int64_t open = __popc(__ballot_sync(0xFFFFFFFFu, lane < D && nres != 0));  // devices occupied to the end
+    r.mk = warp_max((int64_t)end);
+    if (kNarrow && r.mk == 0xFFFFFFFFll) return false;  // (one plus it has wrapped)
+    r.gpu = warp_sum(gsum) + open * r.mk;
+    r.timely = kPhi ? warp_sum(timely) : 0;
+    r.life = kPhi ? warp_sum(life) : 0;
+    r.p95 = (int64_t)(warp_select(LatencyArr<TT>{wm.comp, dp.arrival}, W, p95_rank(W)) ^ (1ull << 63));
+    __syncwarp();  // the memory is free for the next plan
+    return true;
+}
+
+// Plan p's results, by lane 0 (r's makespan counted from 0; first: the first arrival).
+__device__ __forceinline__ void put_result(const wf_dev_problem &dp, const wf_eval_out &out, int64_t p, uint32_t st,
+                                           const PlayResult &r, int64_t first)
+{
+    if ((threadIdx.x & 31) != 0) return;
+    out.status[p] = st;
+    out.makespan_us[p] = st ? WF_INF64 : r.mk - first;
+    out.p95_us[p] = st ? WF_INF64 : r.p95;
+    out.gpu_us[p] = st ? WF_INF64 : r.gpu;
+    if (dp.phi_life) {
+        dp.phi_timely[p] = st ? WF_INF64 : r.timely;
+        dp.phi_life[p] = st ? WF_INF64 : r.life;
     }
 }
 
-// The int64 path for the plans whose times overflow the sweep's u32 slots.
+constexpr size_t kSmemMax = 227 * 1024;
+
+// Every plan of the batch, or (list) the plans whose times a sweep could not
+// hold, on int64 times; a CTA is one warp and walks over plans.  Finish times
+// in shared memory (kShared), else in a row of the context's scratch (windows
+// beyond about 28,000 activations).
+template <bool kShared>
+__global__ void __launch_bounds__(32, 12)
+eval_warp_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
+                 const int32_t *list, const int32_t *count)
+{
+    extern __shared__ __align__(16) uint8_t esm[];
+    const int64_t n = list ? (int64_t)*count : pl.P;
+    uint8_t *big = kShared ? esm + warp_small_bytes(dp.D) : scratch + (size_t)blockIdx.x * row_bytes;
+    const WarpMem<uint64_t> wm = warp_mem<uint64_t>(dp, esm, big);
+    for (int64_t k = blockIdx.x; k < n; k += gridDim.x) {
+        const int64_t p = list ? (int64_t)list[k] : k;
+        const PlanRows pr = plan_rows(pl, p);
+        const uint32_t st = warp_status(dp, pr, (uint16_t *)big);
+        PlayResult r = {};
+        if (!st) {
+            if (dp.phi_life) warp_play<uint64_t, uint64_t, true>(dp, pr, wm, r);
+            else warp_play<uint64_t, uint64_t, false>(dp, pr, wm, r);
+        }
+        put_result(dp, out, p, st, r, dp.first_arrival);
+    }
+}
+
+// The replica batch limit on the int64 path: a thread per plan, rows of
+// global scratch; every plan, or the listed ones.
 __global__ void __launch_bounds__(kEvalThreads)
-eval_list_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
-                 int64_t rows, const int32_t *list, const int32_t *count)
+eval_batched_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
+                    int64_t rows, const int32_t *list, const int32_t *count)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int32_t n = *count;
+    const int64_t n = list ? (int64_t)*count : pl.P;
     if (t >= rows || t >= n) return;
     Row row = row_at(dp, scratch + (size_t)t * row_bytes);
     for (int64_t k = t; k < n; k += rows) {
-        const int64_t p = list[k];
+        const int64_t p = list ? (int64_t)list[k] : k;
         const PlanRows pr = plan_rows(pl, p);
         const uint32_t st = plan_status(dp, pr, row);
         out.status[p] = st;
         if (st) {
             out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
-            if (dp.phi_life) dp.phi_timely[p] = dp.phi_life[p] = WF_INF64;
             continue;
         }
-        int64_t mk, g, phi[2];
-        if (dp.batch > 0) play_batched(dp, pr, row, &mk, &g);
-        else play<false>(dp, pr, row, 0, &mk, &g, dp.phi_life ? phi : nullptr);
+        int64_t mk, g;
+        play_batched(dp, pr, row, &mk, &g);
         out.makespan_us[p] = mk;
         out.gpu_us[p] = g;
         out.p95_us[p] = select_rank(row.comp, dp.W, p95_rank(dp.W));
-        if (dp.phi_life) { dp.phi_timely[p] = phi[0]; dp.phi_life[p] = phi[1]; }
     }
 }
 
@@ -493,7 +723,7 @@ eval_stoch_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scra
         for (int32_t s = threadIdx.x; s < S; s += blockDim.x) {
             const uint64_t key = splitmix(splitmix(dp.seed ^ gp) ^ (uint64_t)s);
             int64_t mk, g;
-            play<true>(dp, pr, row, key, &mk, &g);
+            play(dp, pr, row, key, &mk, &g);
             atomicAdd(&s_mk, (unsigned long long)mk);
             atomicAdd(&s_gpu, (unsigned long long)g);
             for (int32_t w = 0; w < W; ++w) pool[(int64_t)s * W + w] = row.comp[w];
@@ -558,6 +788,38 @@ size_t wf_eval_scratch_bytes(const wf_dev_problem &dp, int64_t max_P, int64_t *u
     return unit * (size_t)*units;
 }
 
+namespace {
+
+// The int64 path over every plan (list null) or the listed ones.
+int launch_int64(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, const int32_t *list, const int32_t *count,
+                 cudaStream_t st)
+{
+    const wf_dev_problem &dp = ctx->dp;
+    uint8_t *scratch = (uint8_t *)ctx->eval_scratch;
+    const int64_t units = std::min<int64_t>(ctx->eval_threads, plans->P);
+    if (dp.batch > 0) {
+        const int64_t blocks = (units + kEvalThreads - 1) / kEvalThreads;
+        eval_batched_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes,
+                                                                      units, list, count);
+    } else {
+        const bool shared = warp_full_bytes<uint64_t>(dp) <= kSmemMax;
+        const size_t smem = shared ? warp_full_bytes<uint64_t>(dp) : warp_small_bytes(dp.D);
+        const auto kernel = shared ? eval_warp_kernel<true> : eval_warp_kernel<false>;
+        const int rc = wf_cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                          (int)smem), "int64 path smem attribute");
+        if (rc) return rc;
+        // A CTA per plan, or (a list, most often empty) about as many as fit
+        // the chip at once; beyond shared memory, a scratch row per CTA.
+        int64_t blocks = plans->P;
+        if (list) blocks = std::min<int64_t>(blocks, (int64_t)ctx->sms * 12);
+        if (!shared) blocks = std::min<int64_t>(blocks, units);
+        kernel<<<(unsigned)blocks, 32, smem, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes, list, count);
+    }
+    return wf_cuda_check(cudaGetLastError(), "int64 pass launch");
+}
+
+}  // namespace
+
 int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, cudaStream_t st)
 {
     const wf_dev_problem &dp = ctx->dp;
@@ -568,17 +830,13 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
     if (dp.batch > 0 && dp.phi_life)
         return wf_set_error(WF_EINVAL, "the window terms of Eq. 12 are not modelled with a replica batch limit");
     if (dp.S == 0) {
-        const int64_t blocks = (units + kEvalThreads - 1) / kEvalThreads;
         // The replica batch limit: its own sweep in shared memory, the int64
         // path for what it hands on (or for everything, when it does not fit).
         const size_t bsm = dp.batch > 0 && !ctx->force_int64 ? wf_batch_smem(dp) : 0;
         if (bsm) {
             int rc = wf_cuda_check(cudaMemsetAsync(ctx->ovf_count, 0, sizeof(int32_t), st), "reset overflow count");
             if (!rc) rc = wf_launch_batch(ctx, plans, out, bsm, ctx->ovf_list, ctx->ovf_count, st);
-            if (rc) return rc;
-            eval_list_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes,
-                                                                       units, ctx->ovf_list, ctx->ovf_count);
-            return wf_cuda_check(cudaGetLastError(), "int64 pass launch");
+            return rc ? rc : launch_int64(ctx, plans, out, ctx->ovf_list, ctx->ovf_count, st);
         }
         const wf_sweep_cfg cfg = ctx->force_int64 || dp.batch > 0 ? wf_sweep_cfg{} : wf_sweep_config(dp);
         if (dp.reclaim && !cfg.smem64)
@@ -633,13 +891,9 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
                 ctx->wide_P = plans->P;
                 ctx->rb_pair = q;
             }
-            eval_list_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch,
-                                                                       ctx->eval_row_bytes, units,
-                                                                       rest, rest_count);
-        } else {
-            eval_det_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch,
-                                                                        ctx->eval_row_bytes, units);
+            return launch_int64(ctx, plans, out, rest, rest_count, st);
         }
+        return launch_int64(ctx, plans, out, nullptr, nullptr, st);
     } else {
         // Per-thread rows of every CTA first, then one completion pool per CTA.
         int64_t *pool = (int64_t *)(scratch + (size_t)units * kSampleThreads * ctx->eval_row_bytes);
@@ -777,34 +1031,31 @@ __global__ void static_link_kernel(uint8_t *s, wf_dev_problem dp, StaticLayout l
     }
 }
 
-// The deterministic evaluation with one scratch row per plan and the first
-// arrival taken from the static header.
-__global__ void __launch_bounds__(kEvalThreads)
+// The deterministic evaluation, a warp (a CTA) per plan, with the first
+// arrival taken from the static header: on u32 times in shared memory
+// (kShared), and on u64 times in the plan's scratch row when those do not
+// hold the plan or the window does not fit.
+template <typename Q, bool kShared>
+__global__ void __launch_bounds__(32, 16)
 eval_static_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *s, StaticLayout l,
                    size_t row_bytes)
 {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= pl.P) return;
+    extern __shared__ __align__(16) uint8_t esm[];
+    const int64_t p = blockIdx.x;
     if ((*(volatile int *)(s + 8) & 0xFF) == kStaticBadTables) {  // nothing is evaluated
-        out.status[p] = WF_ST_TABLES;
-        out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
+        if (threadIdx.x == 0) {
+            out.status[p] = WF_ST_TABLES;
+            out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
+        }
         return;
     }
-    wf_dev_problem d = dp;
-    d.first_arrival = *(const int64_t *)s;
-    Row row = row_at(d, s + l.rows + (size_t)p * row_bytes);
+    uint8_t *row = s + l.rows + (size_t)p * row_bytes, *big = kShared ? esm + warp_small_bytes(dp.D) : row;
     const PlanRows pr = plan_rows(pl, p);
-    const uint32_t st = plan_status(d, pr, row);
-    out.status[p] = st;
-    if (st) {
-        out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
-        return;
-    }
-    int64_t mk, g;
-    play<false>(d, pr, row, 0, &mk, &g);
-    out.makespan_us[p] = mk;
-    out.gpu_us[p] = g;
-    out.p95_us[p] = select_rank(row.comp, d.W, p95_rank(d.W));
+    const uint32_t st = warp_status(dp, pr, (uint16_t *)big);
+    PlayResult r = {};
+    if (!st && !(kShared && warp_play<uint32_t, Q, false>(dp, pr, warp_mem<uint32_t>(dp, esm, big), r)))
+        warp_play<uint64_t, Q, false>(dp, pr, warp_mem<uint64_t>(dp, esm, row), r);
+    put_result(dp, out, p, st, r, *(const int64_t *)s);
 }
 
 // Device address of the static array per device, from the last lookup
@@ -899,8 +1150,14 @@ extern "C" int wf_eval_plans_static(const wf_problem *pb, const wf_plans *pl, co
     static_check_kernel<<<(unsigned)((cspan + 255) / 256), 256, 0, st>>>(s, dp);
     static_count_kernel<<<grid, 256, 0, st>>>(s, dp, l);
     static_link_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(s, dp, l);
-    eval_static_kernel<<<(unsigned)((pl->P + kEvalThreads - 1) / kEvalThreads), kEvalThreads, 0, st>>>(
-        dp, *pl, *out, s, l, row);
+    const bool shared = warp_full_bytes<uint32_t>(dp) <= kSmemMax;
+    const size_t smem = shared ? warp_full_bytes<uint32_t>(dp) : warp_small_bytes(D);
+    const auto kernel = M <= 8 ? (shared ? eval_static_kernel<uint32_t, true> : eval_static_kernel<uint32_t, false>)
+                               : (shared ? eval_static_kernel<uint64_t, true> : eval_static_kernel<uint64_t, false>);
+    rc = wf_cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                       "static evaluation smem attribute");
+    if (rc) return rc;
+    kernel<<<(unsigned)pl->P, 32, smem, st>>>(dp, *pl, *out, s, l, row);
     return wf_cuda_check(cudaGetLastError(), "static evaluation launch");
 }
 

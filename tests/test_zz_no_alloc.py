@@ -130,3 +130,35 @@ def test_static_entry_reports_tables_that_fail_its_device_check():
     want = oracle.eval_plans(w.problem, plans)
     for a, b in zip(out.numpy(), want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("sessions,sizes,D,M,scale", [(1, (4, 4), 1, 1, 1), (8, (4, 4), 3, 8, 1), (11, (3, 3), 32, 9, 1),
+                                                      (70, (4, 9), 9, 16, 1), (40, (4, 9), 3, 4, 150000), (3, (5, 9), 2, 3, 1 << 24)])
+def test_static_entry_on_edges(sessions, sizes, D, M, scale):
+    """Windows of 32 and 33 activations, both queue words, more than 32
+    sessions, and run times that leave 32 bits for all or some plans (the
+    64-bit replay), against the oracle."""
+    from randprob import random_problem
+    from paper_2609_03335_gb300 import build, wf
+    build.build()
+    rng = np.random.default_rng(sessions * 100 + D)
+    prob = random_problem(rng, n_sessions=sessions, sizes=sizes, D=D, M=M) if sizes != (3, 3) else \
+        random_problem(rng, n_sessions=8, sizes=(4, 4), D=D, M=M)
+    if sizes == (3, 3):  # 33 activations
+        assert prob.N == 32
+        prob = prob.with_(N=33, W=9, pred_off=np.append(prob.pred_off, prob.pred_off[-1]).astype(np.int32),
+                          model=np.append(prob.model, 0).astype(np.uint8), session=np.append(prob.session, 8).astype(np.int32),
+                          arrival_us=np.append(prob.arrival_us, 7), lat_us=np.append(prob.lat_us, np.full(D, 9, np.int32)),
+                          peak_mib=np.append(prob.peak_mib, np.full(D, prob.weight_mib[0] + 1, np.int32)))
+    prob = prob.with_(lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, 2**31 - 1).astype(np.int32))
+    plans = wfgen.make_plans(prob, 300, 5, p_retain=0.7)
+    plans.place[2, 0] = prob.D
+    plans.order[4, 0] = plans.order[4, 1]
+    out = wf.Results(plans.P)
+    wf.wf_eval_plans_static(wf.DeviceProblem(prob), wf.DevicePlans.from_host(plans, "cuda"), out)
+    wf.wf_static_status()
+    want = oracle.eval_plans(prob, plans)
+    if scale > 1:
+        assert want[0][want[3] == 0].max() > 1 << 32
+    for a, b in zip(out.numpy(), want):
+        assert np.array_equal(a, b)
