@@ -830,18 +830,19 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
     if (dp.batch > 0 && dp.phi_life)
         return wf_set_error(WF_EINVAL, "the window terms of Eq. 12 are not modelled with a replica batch limit");
     if (dp.S == 0) {
-        // The replica batch limit: its own sweep in shared memory, the int64
-        // path for what it hands on (or for everything, when it does not fit).
-        const size_t bsm = dp.batch > 0 && !ctx->force_int64 ? wf_batch_smem(dp) : 0;
-        if (bsm) {
-            int rc = wf_cuda_check(cudaMemsetAsync(ctx->ovf_count, 0, sizeof(int32_t), st), "reset overflow count");
-            if (!rc) rc = wf_launch_batch(ctx, plans, out, bsm, ctx->ovf_list, ctx->ovf_count, st);
-            return rc ? rc : launch_int64(ctx, plans, out, ctx->ovf_list, ctx->ovf_count, st);
+        // The replica batch limit has a sweep of its own.  Windows that no
+        // sweep holds play on the int64 path.
+        wf_batch_cfg bcfg = {};
+        wf_sweep_cfg cfg = {};
+        if (!ctx->force_int64) {
+            if (dp.batch > 0) bcfg = wf_batch_config(dp);
+            else cfg = wf_sweep_config(dp);
         }
-        const wf_sweep_cfg cfg = ctx->force_int64 || dp.batch > 0 ? wf_sweep_cfg{} : wf_sweep_config(dp);
+        const bool batch = bcfg.smem64 != 0;
+        const bool narrow = batch || cfg.smem32, wide = batch || cfg.smem64;
         if (dp.reclaim && !cfg.smem64)
             return wf_set_error(WF_EINVAL, "reclamation by next use runs only in the shared-memory sweep");
-        if (cfg.smem32 || cfg.smem64) {
+        if (narrow || wide) {
             // Under stream capture (a CUDA graph) nothing but launches on the
             // stream may happen: the path choice stays as it is.
             cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -861,7 +862,7 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
                     return wf_cuda_check(q, "overflow count event");
                 }
             }
-            const bool wide_first = (ctx->prefer_wide || ctx->start_path >= WF_PATH_WIDE) && cfg.smem64;
+            const bool wide_first = (ctx->prefer_wide || ctx->start_path >= WF_PATH_WIDE) && wide;
             // Two pairs of counts, taken by calls in turn, so that a call
             // issued before an earlier call's read-back has run does not
             // reset the count it reads; a call that comes back to a pair
@@ -873,10 +874,13 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
                 rc = wf_cuda_check(cudaStreamWaitEvent(st, ctx->ovf_event, 0), "overflow read-back wait");
             if (!rc) rc = wf_cuda_check(cudaMemsetAsync(counts, 0, 2 * sizeof(int32_t), st), "reset overflow counts");
             const int32_t *rest = nullptr, *rest_count = nullptr;
-            if (!rc) rc = wf_launch_sweep(ctx, plans, out, cfg, wide_first, counts, ctx->ovf_list, ctx->ovf_list2, st,
-                                          &rest, &rest_count);
+            if (!rc)
+                rc = batch ? wf_launch_batch(ctx, plans, out, bcfg, wide_first, counts, ctx->ovf_list, ctx->ovf_list2, st,
+                                             &rest, &rest_count)
+                           : wf_launch_sweep(ctx, plans, out, cfg, wide_first, counts, ctx->ovf_list, ctx->ovf_list2, st,
+                                             &rest, &rest_count);
             if (rc) return rc;
-            if (cfg.smem32 && !wide_first && !ctx->wide_pending && !capturing) {
+            if (narrow && !wide_first && !ctx->wide_pending && !capturing) {
                 // The read-back runs on the context's side stream after the
                 // sweeps, so the caller's stream never waits for it; the
                 // value only picks the path, never a result.

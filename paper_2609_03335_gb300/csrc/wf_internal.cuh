@@ -61,7 +61,7 @@ struct wf_dev_problem {
     uint16_t *nextuse;
     // Replica batch limit B_q (wf_ctx_set_batch): 0 = one unit at a time per
     // device (the sweeps); >= 1 = up to B_q units of a device's current
-    // replica at once, played by the int64 path.
+    // replica at once, played by a sweep of their own (wf_batch.cu).
     int32_t batch;
     int64_t max_chain_run;      // the longest fusible chain's run time on its slowest devices, plus the grant
     // Outputs of the window terms of Eq. 12 ([P] each, wf_eval_plans_phi);
@@ -167,9 +167,16 @@ int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, c
 size_t wf_stoch_smem(const wf_dev_problem &dp);
 // The status pass (place false: the sweep's producers check the placement).
 int wf_launch_status(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st, bool place);
-size_t wf_batch_smem(const wf_dev_problem &dp);
-int wf_launch_batch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, size_t smem, int32_t *ovf_list,
-                    int32_t *ovf_count, cudaStream_t st);
+// The replica-batch sweep on u32 and on u64 times (shared memory of a CTA; 0
+// = not usable).
+struct wf_batch_cfg {
+    size_t smem32;
+    size_t smem64;
+};
+wf_batch_cfg wf_batch_config(const wf_dev_problem &dp);
+int wf_launch_batch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, const wf_batch_cfg &cfg, bool wide_first,
+                    int32_t *counts, int32_t *list1, int32_t *list2, cudaStream_t st, const int32_t **rest_list,
+                    const int32_t **rest_count);
 int wf_launch_stoch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, size_t smem,
                     int32_t *ovf_list, int32_t *ovf_count, cudaStream_t st);
 // Status pass, then the sweeps (u32 first unless wide_first; then the

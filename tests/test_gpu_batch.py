@@ -1,5 +1,6 @@
-"""GPU parity for the replica batch limit B_q (wf_ctx_set_batch): the int64
-path's batched play against the oracle's, element by element."""
+"""GPU parity for the replica batch limit B_q (wf_ctx_set_batch): the replica
+batch sweep and the int64 path's batched play against the oracle's, element by
+element."""
 import numpy as np
 import pytest
 
@@ -59,12 +60,40 @@ def test_burst_window_in_full(B):
 
 
 def test_batch_one_equals_the_sweep():
-    """B_q = 1 on the int64 path gives the shared-memory sweep's results."""
+    """B_q = 1 gives the results of the sweep without a limit."""
     w = wfgen.config("mix")
     plans = wfgen.make_plans(w.problem, 8192, 4)
     a = gpu_eval(w.problem, plans)
     b = _gpu(w.problem.with_(batch=1), plans)
     assert_same(b, a)
+
+
+@pytest.mark.parametrize("D,M,B,P", [(1, 1, 1, 1), (8, 8, 4, 65), (8, 9, 5, 7), (9, 8, 4, 33), (16, 16, 64, 9),
+                                     (17, 8, 3, 8), (32, 16, 5, 17)])
+def test_lanes_per_plan(D, M, B, P):
+    """8, 16 and 32 lanes per plan, both queue words, running slots in
+    registers and in shared memory, CTAs whose plans are not all there."""
+    rng = np.random.default_rng(10 * D + B)
+    prob = random_problem(rng, n_sessions=40, D=D, M=M).with_(batch=B)
+    plans = wfgen.make_plans(prob, P, 3, p_retain=0.6 if B == 1 else None)
+    assert_same(_gpu(prob, plans), oracle_eval(prob, plans))
+
+
+@pytest.mark.parametrize("scale,B", [(165000, 2), (1 << 20, 4), (1 << 20, 6), (1 << 24, 1)])
+def test_times_past_32_bits(scale, B):
+    """Some or all plans leave the 32-bit sweep (and with the largest scale
+    some fused chains' run times too): the 64-bit sweep and the int64 path,
+    twice on one context (the second call may start on 64-bit times)."""
+    wf = lib()
+    rng = np.random.default_rng(scale % 97 + B)
+    prob = random_problem(rng, n_sessions=30, sizes=(6, 12), D=4, M=5)
+    prob = prob.with_(batch=B, lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, 2**31 - 1).astype(np.int32))
+    plans = wfgen.make_plans(prob, 200, 6)
+    want = oracle_eval(prob, plans)
+    ctx = wf.Ctx(prob, max_P=plans.P)
+    for _ in range(2):
+        assert_same(gpu_eval(prob, plans, ctx=ctx), want)
+    ctx.close()
 
 
 def test_refusals():
