@@ -144,6 +144,118 @@ struct PairArr {
     }
 };
 
+// Residency of one device under least-recently-used reclamation in one
+// shared-memory word: the queue of 4-bit model ids, least recently used in
+// nibble 0, empty places 0xF, and the free capacity (capacity minus resident
+// weights); up to 8 models the queue says its own length (no id has bit 3
+// set), beyond it is kept beside.  settle() plays a unit's admission (Eq. 11,
+// Section 3.5): the unit's own model leaves the queue first, the victims are
+// then its first entries, and the model goes back in last.  The first three
+// victims' weights are read at once and taken without branching (a loop over
+// victims waited for one weight at a time: about 130 instructions a unit with
+// it, half of that without).  Returns the record's rewritten (w1, w3): the
+// load the unit waits for (none on a hit, Eq. 5) and the occupancy changes.
+template <typename Q>
+struct DevState;
+
+// The victims: from `need` and the free capacity f, the shift that drops the
+// evicted entries from queue q (at most n4 / 4 of them).
+template <typename Q>
+__device__ __forceinline__ int evict(Q q, uint32_t need, uint32_t &f, int n4, const int32_t *weight)
+{
+    const uint32_t w0 = (uint32_t)weight[(uint32_t)q & 15u], w1 = (uint32_t)weight[(uint32_t)(q >> 4) & 15u],
+                   w2 = (uint32_t)weight[(uint32_t)(q >> 8) & 15u];
+    int e4 = 0;
+    if (need > f) { f += w0; e4 = 4; }
+    if (need > f) { f += w1; e4 = 8; }
+    if (need > f) { f += w2; e4 = 12; }
+    for (; need > f && e4 < n4; e4 += 4) f += (uint32_t)weight[(uint32_t)(q >> e4) & 15u];
+    return min(e4, n4);
+}
+
+__device__ __forceinline__ uint2 settled(uint32_t r3, bool hit, uint32_t ld, bool was_empty, bool emptied)
+{
+    return make_uint2(hit ? 0u : ld, (r3 & ~(hit ? kPrefetch | kWasEmpty : kWasEmpty)) | (was_empty ? kWasEmpty : 0u) |
+                                         (emptied ? kEmptied : 0u));
+}
+
+template <>
+struct DevState<uint32_t> {
+    uint2 v;  // queue, free capacity
+    __device__ __forceinline__ void init(uint32_t cap) { v = make_uint2(~0u, cap); }
+    __device__ __forceinline__ bool occupied() const { return v.x != ~0u; }
+    __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
+                                            int32_t D, int *err, bool &missed)
+    {
+        const uint32_t m = (r3 >> 5) & 15u, wm = (uint32_t)weight[m], ld = (uint32_t)load[m * D + (r3 & 31u)];
+        uint32_t q = v.x, f = v.y;
+        const bool was_empty = q == ~0u;
+        const uint32_t x = q ^ (0x11111111u * m);
+        const uint32_t z = (x - 0x11111111u) & ~x & 0x88888888u;  // its lowest bit: the nibble equal to m
+        const bool hit = z != 0;
+        missed = !hit;
+        const uint32_t below = ((z & (0u - z)) >> 3) - 1u;  // the bits below that nibble (all when there is none)
+        q = (q & below) | ((q >> 4) & ~below) | 0xF0000000u;
+        const uint32_t need = hit ? r1 : wm + r1;  // at most the capacity
+        const int e4 = evict(q, need, f, 32, weight);
+        if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
+        q = __funnelshift_rc(q, ~0u, e4);
+        const uint32_t gap = q & 0x88888888u;
+        const uint32_t at = (gap & (0u - gap)) >> 3;  // 1 << 4 n: the first empty place
+        const uint32_t with = q - (15u - m) * at;     // 0xF there becomes m
+        f -= hit ? 0u : wm;
+        bool emptied = false;
+        if (r3 & kDrop) {  // the model leaves when the unit ends
+            f += wm;
+            emptied = q == ~0u;
+        } else {
+            q = with;
+        }
+        v = make_uint2(q, f);
+        return settled(r3, hit, ld, was_empty, emptied);
+    }
+};
+
+template <>
+struct DevState<uint64_t> {
+    uint4 v;  // queue (low, high), free capacity, models held
+    __device__ __forceinline__ void init(uint32_t cap) { v = make_uint4(~0u, ~0u, cap, 0u); }
+    __device__ __forceinline__ bool occupied() const { return v.w != 0; }
+    __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
+                                            int32_t D, int *err, bool &missed)
+    {
+        const uint32_t m = (r3 >> 5) & 15u, wm = (uint32_t)weight[m], ld = (uint32_t)load[m * D + (r3 & 31u)];
+        uint64_t q = ((uint64_t)v.y << 32) | v.x;
+        uint32_t f = v.z, n = v.w;
+        const bool was_empty = n == 0;
+        const uint64_t x = q ^ (0x1111111111111111ull * m);
+        const uint64_t z = (x - 0x1111111111111111ull) & ~x & 0x8888888888888888ull;
+        const uint64_t low = (z & (0ull - z)) >> 3;
+        // (with 16 models the empty places match the last one)
+        const bool hit = low != 0 && (uint32_t)__popcll(low - 1) < 4 * n;
+        missed = !hit;
+        const uint64_t below = hit ? low - 1 : ~0ull;
+        q = (q & below) | ((q >> 4) & ~below) | (hit ? 0xFull << 60 : 0ull);
+        n -= hit ? 1u : 0u;
+        const uint32_t need = hit ? r1 : wm + r1;
+        const int e4 = evict(q, need, f, (int)(4 * n), weight);
+        if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
+        q = e4 < 64 ? (q >> e4) | ~(~0ull >> e4) : ~0ull;
+        n -= (uint32_t)e4 >> 2;
+        f -= hit ? 0u : wm;
+        bool emptied = false;
+        if (r3 & kDrop) {
+            f += wm;
+            emptied = n == 0;
+        } else {
+            q ^= (uint64_t)(15u ^ m) << (4 * n);
+            n += 1;
+        }
+        v = make_uint4((uint32_t)q, (uint32_t)(q >> 32), f, n);
+        return settled(r3, hit, ld, was_empty, emptied);
+    }
+};
+
 struct PcLayout {
     uint32_t weight, cap, load, arr, ring, slots, slots_hi, tfree, used, queue, nres, open, flag, nuse, rcnt, gmask,
         everl, total;
@@ -161,7 +273,7 @@ __host__ __device__ inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, i
     constexpr uint32_t t = sizeof(TT);
     PcLayout l;
     uint32_t o = 0;
-    l.weight = o; o += round16(4u * M);
+    l.weight = o; o += 4u * 16;  // (zeros beyond M: read for the queue's empty places)
     l.cap = o; o += round16(4u * D);
     l.load = o; o += round16(4u * M * D);
     l.arr = o; o += round16(4u * W);
@@ -170,9 +282,11 @@ __host__ __device__ inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, i
     l.slots_hi = o; o += round16(SlotBytes<ST>::kHi * (uint32_t)NS * kP);
     l.tfree = o; o += round16(t * D * kP);
     const uint32_t rs = (uint32_t)(PcGroups<kP, kReclaim>::rows(D) * PcGroups<kP, kReclaim>::kLanes);
-    l.used = o; o += round16(4u * rs);
-    l.queue = o; o += round16((M <= 8 ? 4u : 8u) * rs);  // Lru<uint32_t> or Lru<uint64_t>
-    l.nres = o; o += round16(rs);
+    // Residency state: a word per device (DevState), or under reclamation by
+    // next use weights, queue and count apart.
+    l.queue = o; o += round16((kReclaim ? (M <= 8 ? 4u : 8u) : (M <= 8 ? 8u : 16u)) * rs);
+    l.used = o; o += kReclaim ? round16(4u * rs) : 0u;
+    l.nres = o; o += kReclaim ? round16(rs) : 0u;
     l.open = o; o += round16(4u * kP);
     l.flag = o; o += 16;
     l.nuse = o; o += kReclaim ? round16(2u * D * M * kP) : 0u;
@@ -301,7 +415,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     uint32_t *arrival = (uint32_t *)(sm + L.arr);
     uint32_t *open = (uint32_t *)(sm + L.open);
     uint32_t *gmask = (uint32_t *)(sm + L.gmask);  // [buffer][device group][plan]
-    for (int32_t k = threadIdx.x; k < M; k += blockDim.x) weight[k] = __ldg(dp.weight + k);
+    if (threadIdx.x < 16) weight[threadIdx.x] = (int)threadIdx.x < M ? __ldg(dp.weight + threadIdx.x) : 0;
     for (int32_t k = threadIdx.x; k < D; k += blockDim.x) cap[k] = __ldg(dp.cap + k);
     for (int32_t k = threadIdx.x; k < M * D; k += blockDim.x) load[k] = __ldg(dp.load + k);
     for (int32_t k = threadIdx.x; k < W; k += blockDim.x) arrival[k] = (uint32_t)__ldg(dp.arrival + k);
@@ -412,15 +526,17 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         const int64_t p = (rmine && qp < ng) ? (in_list ? (int64_t)in_list[j0 + qp] : j0 + qp) : 0;
         const bool live = rmine && qp < ng && out.status[p] == 0;
         constexpr int kRow = PcGroups<kP, kReclaim>::kLanes;
-        uint32_t *used = (uint32_t *)(sm + L.used) + rl;  // [device / kG][lane]
+        uint32_t *used = (uint32_t *)(sm + L.used) + rl;  // [device / kG][lane] (reclamation by next use)
         Q *queue = (Q *)(sm + L.queue) + rl;
         uint8_t *nres = sm + L.nres + rl;
+        DevState<Q> *state = (DevState<Q> *)(sm + L.queue) + rl;  // [device / kG][lane] (least recently used)
         uint16_t *nuse = (uint16_t *)(sm + L.nuse) + qp;  // [device][model][plan]
         uint8_t *rcnt = sm + L.rcnt + qp;                 // [model][plan]
         uint16_t *everl = (uint16_t *)(sm + L.everl) + rl;  // [device / kG][lane], bit m: m was held (kPhi)
         if (rmine) {
             for (int32_t t = 0; t * kG + g < D; ++t) {
-                used[t * kRow] = 0; queue[t * kRow] = 0; nres[t * kRow] = 0;
+                if (kReclaim) { used[t * kRow] = 0; queue[t * kRow] = 0; nres[t * kRow] = 0; }
+                else state[t * kRow].init((uint32_t)__ldg(dp.cap + t * kG + g));
                 if (kPhi) everl[t * kRow] = 0;
             }
             if (kReclaim)
@@ -444,19 +560,15 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 const int32_t d = (int32_t)(r3 & 31u);
                 if (!kReclaim) {
                     const int32_t t = d / kG;
-                    Q q = queue[t * kRow];
-                    uint32_t n = nres[t * kRow];
-                    uint32_t u_d = used[t * kRow];
+                    DevState<Q> ds = state[t * kRow];
                     bool missed;
-                    uint2 w = settle_lru<Q>(q, n, u_d, (uint32_t)cap[d], r1, r3, weight, load, D, dp.err, missed);
+                    uint2 w = ds.settle(r1, r3, weight, load, D, dp.err, missed);
                     if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
                         const uint32_t m = (r3 >> 5) & 15u, e = everl[t * kRow];
                         w.x |= ((e >> m) & 1u) << 31;
                         everl[t * kRow] = (uint16_t)(e | (1u << m));
                     }
-                    queue[t * kRow] = q;
-                    nres[t * kRow] = (uint8_t)n;
-                    used[t * kRow] = u_d;
+                    state[t * kRow] = ds;
                     rb[(1 * kChunk + k) * kPitch] = w;
                 } else {
                     // Reclamation by next use: victims one at a time, a copy
@@ -542,7 +654,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         }
         if (live) {  // devices still occupied at the end
             uint32_t o = 0;
-            for (int32_t t = 0; t * kG + g < D; ++t) o += nres[t * kRow] != 0;
+            for (int32_t t = 0; t * kG + g < D; ++t) o += kReclaim ? nres[t * kRow] != 0 : state[t * kRow].occupied();
             if (o) atomicAdd(open + qp, o);
         }
         named_arrive(kOpen, kResThreads + 32);
