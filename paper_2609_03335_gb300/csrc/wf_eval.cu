@@ -901,10 +901,9 @@ int wf_launch_eval(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, c
     } else {
         // Per-thread rows of every CTA first, then one completion pool per CTA.
         int64_t *pool = (int64_t *)(scratch + (size_t)units * kSampleThreads * ctx->eval_row_bytes);
-        const size_t smem = ctx->force_int64 ? 0 : wf_stoch_smem(dp);
-        if (smem) {
+        if (!ctx->force_int64 && wf_stoch_usable(dp)) {
             int rc = wf_cuda_check(cudaMemsetAsync(ctx->ovf_count, 0, sizeof(int32_t), st), "reset overflow count");
-            if (!rc) rc = wf_launch_stoch(ctx, plans, out, smem, ctx->ovf_list, ctx->ovf_count, st);
+            if (!rc) rc = wf_launch_stoch(ctx, plans, out, ctx->ovf_list, ctx->ovf_count, st);
             if (rc) return rc;
             const int64_t lunits = std::min<int64_t>(units, (int64_t)ctx->sms * 4);
             eval_stoch_kernel<<<(unsigned)lunits, kSampleThreads, 0, st>>>(dp, *plans, *out, scratch,

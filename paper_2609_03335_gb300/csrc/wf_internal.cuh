@@ -164,7 +164,8 @@ struct wf_sweep_cfg {
 };
 wf_sweep_cfg wf_sweep_config(const wf_dev_problem &dp);
 int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st);
-size_t wf_stoch_smem(const wf_dev_problem &dp);
+// The stochastic sweep (wf_stoch.cu) holds this problem.
+bool wf_stoch_usable(const wf_dev_problem &dp);
 // The status pass (place false: the sweep's producers check the placement).
 int wf_launch_status(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st, bool place);
 // The replica-batch sweep on u32 and on u64 times (shared memory of a CTA; 0
@@ -177,8 +178,8 @@ wf_batch_cfg wf_batch_config(const wf_dev_problem &dp);
 int wf_launch_batch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, const wf_batch_cfg &cfg, bool wide_first,
                     int32_t *counts, int32_t *list1, int32_t *list2, cudaStream_t st, const int32_t **rest_list,
                     const int32_t **rest_count);
-int wf_launch_stoch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, size_t smem,
-                    int32_t *ovf_list, int32_t *ovf_count, cudaStream_t st);
+int wf_launch_stoch(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, int32_t *ovf_list, int32_t *ovf_count,
+                    cudaStream_t st);
 // Status pass, then the sweeps (u32 first unless wide_first; then the
 // relative sweep where it applies and the context's path is not
 // WF_PATH_WIDE, else u64); on return *rest_list / *rest_count name the plans
