@@ -47,7 +47,7 @@ namespace {
 // slots need the room.
 constexpr int kPlans32 = 16;                // plans per CTA of the u32 sweep
 // Record buffers of the ring: four, or three under reclamation by next use,
-// whose seventh record word would otherwise cost a CTA per SM at 2,000
+// whose state per model would otherwise cost a CTA per SM at 2,000
 // activations.  Named barriers: kFullP + b (producers -> residency), kFullR +
 // b (residency -> timing), kEmpty + b (timing -> producers) for buffer b;
 // kOpen (residency -> timing, once at the end).
@@ -60,20 +60,25 @@ struct Ring {
 
 // The ring holds a record as word pairs (8-byte shared-memory accesses):
 // (w0, w2) for timing, (w1, w3) read and rewritten by residency, (w4, w5)
-// for timing, and under reclamation by next use (the unit's next use, 0).
-template <int kReclaim>
-struct RecPairs {
-    static constexpr int kPairs = 3 + kReclaim;
-};
+// for timing; under reclamation by next use the unit's next use is beside it
+// (u16: as a fourth pair it cost a CTA per SM at 2,000 activations).
+constexpr int kPairs = 3;
 
-template <int kP>
+// Lanes per plan of the residency stage under reclamation by next use: kPer
+// models a lane, of the 8 or 16 that a sweep is compiled for.
+template <typename Q>
+constexpr int kPer = sizeof(Q) == 4 ? 1 : 2;
+template <typename Q>
+constexpr int kModelLanes = 2 * (int)sizeof(Q) / kPer<Q>;
+
+template <int kP, int kReclaim = 0, typename Q = uint32_t>
 struct PcShape {
     static constexpr int kProducers = kP >= 32 ? 8 : kP >= 16 ? 4 : kP >= 6 ? 3 : 2;
-    static constexpr int kRes = kP >= 32 ? 4 : kP >= 16 ? 2 : 1;  // residency warps
+    static constexpr int kRes = kReclaim ? (kP * kModelLanes<Q> + 31) / 32 : kP >= 32 ? 4 : kP >= 16 ? 2 : 1;  // residency warps
     static constexpr int kWarps = 1 + kRes + kProducers;
     // Four 16-plan CTAs share an SM (shared memory allows it at 2,000
     // activations), which bounds the registers per thread.
-    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP >= 16 ? 4 : 1;
+    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP < 16 ? 1 : kReclaim && sizeof(Q) == 8 ? 3 : 4;
     // Elements (8-byte word pairs) per (pair, position) row of the ring.  A
     // producer store covers 16 positions x 2 plans in two halves of 16
     // lanes; an odd pitch puts each half's 16 pairs on 32 distinct banks, and
@@ -82,15 +87,17 @@ struct PcShape {
     static_assert(kChunk == 16 && kP >= 1 && kP <= 32, "ring pitch assumes 16 positions per chunk");
 };
 
-// Residency lanes per plan: a device group each (d = g mod kG), or one lane
-// for every device under reclamation by next use.
-// A lane's state for its t-th device (d = g + t kG) sits at [t][lane]: the
-// lanes of a warp touch consecutive words.
-template <int kP, int kReclaim>
+// Residency lanes per plan under least-recently-used reclamation: a device
+// group each (d = g mod kG).  A lane's state for its t-th device (d = g + t kG)
+// sits at [t][lane]: the lanes of a warp touch consecutive words.  Under
+// reclamation by next use the lanes are a plan's models, every device is
+// played by all of them (one group), and the state is [device][lane].
+template <int kP, int kReclaim, typename Q>
 struct PcGroups {
-    static constexpr int kG = kReclaim ? 1 : (32 * PcShape<kP>::kRes) / kP;
-    static constexpr int kLanes = kG == 1 ? kP : 32 * PcShape<kP>::kRes;  // row length of the state
-    static_assert(kG >= 1 && kG * kP <= 32 * PcShape<kP>::kRes, "residency lanes");
+    using S = PcShape<kP, kReclaim, Q>;
+    static constexpr int kG = kReclaim ? 1 : (32 * S::kRes) / kP;
+    static constexpr int kLanes = 32 * S::kRes;  // row length of the state
+    static_assert(kG >= 1 && kG * kP <= 32 * S::kRes, "residency lanes");
     __host__ __device__ static int32_t rows(int32_t D) { return (D + kG - 1) / kG; }
 };
 
@@ -252,44 +259,50 @@ struct DevState<uint64_t> {
 };
 
 struct PcLayout {
-    uint32_t weight, cap, load, arr, ring, slots, slots_hi, tfree, used, queue, nres, open, flag, nuse, rcnt, gmask,
-        everl, total;
+    uint32_t weight, load, rcost, wsum, arr, ring, next, slots, slots_hi, tfree, free, queue, open, flag, gmask, everl, total;
 };
 
 // Shared memory of a CTA of kP plans with TT times and NS slots per plan;
-// with reclamation by next use (kReclaim) the ring carries a seventh record
-// word and each plan keeps per (device, model) the next use of the resident
-// copy and per model the number of devices holding it; with the window terms
-// of Eq. 12 (kPhi) each residency lane keeps per device the models it ever
-// held.
-template <int kP, typename TT, int kReclaim = 0, bool kPhi = false, typename ST = TT>
-__host__ __device__ inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, int32_t NS)
+// with reclamation by next use (kReclaim) the next uses lie beside the ring
+// and each plan keeps per (device, model) the next use and the last use
+// of the resident copy, and per device the free capacity; with the window
+// terms of Eq. 12 (kPhi) each residency lane keeps per device the models it
+// ever held (by next use: in a register, per model the devices).
+template <int kP, typename TT, typename Q, int kReclaim = 0, bool kPhi = false, typename ST = TT>
+__host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W, int32_t NS)
 {
+    using G = PcGroups<kP, kReclaim, Q>;
     constexpr uint32_t t = sizeof(TT);
     PcLayout l;
     uint32_t o = 0;
     l.weight = o; o += 4u * 16;  // (zeros beyond M: read for the queue's empty places)
-    l.cap = o; o += round16(4u * D);
     l.load = o; o += round16(4u * M * D);
+    l.rcost = o; o += kReclaim ? round16(4u * M * D) : 0u;
+    l.wsum = o; o += kReclaim ? 256u * (uint32_t)sizeof(Q) : 0u;  // (256 sums for each eight models)
     l.arr = o; o += round16(4u * W);
-    l.ring = o; o += round16(8u * Ring<kReclaim>::kBuffers * RecPairs<kReclaim>::kPairs * kChunk * PcShape<kP>::kPitch);
+    l.ring = o; o += round16(8u * Ring<kReclaim>::kBuffers * kPairs * kChunk * PcShape<kP>::kPitch);
+    l.next = o; o += kReclaim ? round16(2u * Ring<kReclaim>::kBuffers * kChunk * PcShape<kP>::kPitch) : 0u;
     l.slots = o; o += round16(SlotBytes<ST>::kLo * (uint32_t)NS * kP);
     l.slots_hi = o; o += round16(SlotBytes<ST>::kHi * (uint32_t)NS * kP);
     l.tfree = o; o += round16(t * D * kP);
-    const uint32_t rs = (uint32_t)(PcGroups<kP, kReclaim>::rows(D) * PcGroups<kP, kReclaim>::kLanes);
+    const uint32_t rs = (uint32_t)(G::rows(D) * G::kLanes);
     // Residency state: a word per device (DevState), or under reclamation by
-    // next use weights, queue and count apart.
-    l.queue = o; o += round16((kReclaim ? (M <= 8 ? 4u : 8u) : (M <= 8 ? 8u : 16u)) * rs);
-    l.used = o; o += kReclaim ? round16(4u * rs) : 0u;
-    l.nres = o; o += kReclaim ? round16(rs) : 0u;
+    // next use a word per (device, model), and the free capacity apart.
+    l.queue = o; o += round16((kReclaim ? 4u * kPer<Q> : (uint32_t)sizeof(DevState<Q>)) * rs);
+    l.free = o; o += kReclaim ? round16(4u * D * kP) : 0u;
     l.open = o; o += round16(4u * kP);
     l.flag = o; o += 16;
-    l.nuse = o; o += kReclaim ? round16(2u * D * M * kP) : 0u;
-    l.rcnt = o; o += kReclaim ? round16((uint32_t)M * kP) : 0u;
-    l.gmask = o; o += round16(4u * Ring<kReclaim>::kBuffers * PcGroups<kP, kReclaim>::kG * kP);
-    l.everl = o; o += kPhi ? round16(2u * rs) : 0u;
+    l.gmask = o; o += kReclaim ? 0u : round16(4u * Ring<kReclaim>::kBuffers * G::kG * kP);
+    l.everl = o; o += kPhi && !kReclaim ? round16(2u * rs) : 0u;
     l.total = o;
     return l;
+}
+
+template <int kP, typename TT, int kReclaim = 0, bool kPhi = false, typename ST = TT>
+inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, int32_t NS)
+{
+    return M <= 8 ? pc_layout_q<kP, TT, uint32_t, kReclaim, kPhi, ST>(D, M, W, NS)
+                  : pc_layout_q<kP, TT, uint64_t, kReclaim, kPhi, ST>(D, M, W, NS);
 }
 
 
@@ -320,19 +333,19 @@ __device__ TT select_slots(const SA &v, int32_t n, int32_t r)
 // TT = uint64_t: only a unit whose summed run time reaches 2^32 - 1 sends its
 // plan to ovf_list.
 template <typename Q, typename TT, int kP, int kReclaim, bool kPhi, typename ST>
-__global__ void __launch_bounds__(32 * PcShape<kP>::kWarps, PcShape<kP>::kMinBlocks)
+__global__ void __launch_bounds__(32 * PcShape<kP, kReclaim, Q>::kWarps, PcShape<kP, kReclaim, Q>::kMinBlocks)
 pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_list, const int32_t *in_count,
           int32_t *ovf_list, int32_t *ovf_count)
 {
-    constexpr int kRW = RecPairs<kReclaim>::kPairs;  // word pairs per record in the ring
-    using S = PcShape<kP>;
+    constexpr int kRW = kPairs;  // word pairs per record in the ring
+    using S = PcShape<kP, kReclaim, Q>;
     constexpr int kPitch = S::kPitch;
     constexpr int kProdThreads = 32 * S::kProducers;
     constexpr int kResThreads = 32 * S::kRes;
     constexpr bool kNarrow = sizeof(TT) == 4;
     constexpr bool kRel = IsRel<ST>::value;  // relative 32-bit times
     static_assert(!kRel || (kNarrow && kReclaim == 0 && !kPhi), "relative times: u32, least recently used");
-    constexpr int kG = PcGroups<kP, kReclaim>::kG;  // residency lanes per plan
+    constexpr int kG = PcGroups<kP, kReclaim, Q>::kG;  // residency lanes per plan (by next use: one mask for all of them)
     using RG = Ring<kReclaim>;
     constexpr int kBuffers = RG::kBuffers, kFullP = RG::kFullP, kFullR = RG::kFullR, kEmpty = RG::kEmpty,
                   kOpen = RG::kOpen;
@@ -340,22 +353,31 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t N = dp.N, D = dp.D, M = dp.M, W = dp.W;
     const int32_t rank = (int32_t)((95 * (int64_t)W + 99) / 100 - 1);  // the p95's nearest rank (Section 4.2)
-    const PcLayout L = pc_layout<kP, TT, kReclaim, kPhi, ST>(D, M, W, dp.nslots + 2);
+    const PcLayout L = pc_layout_q<kP, TT, Q, kReclaim, kPhi, ST>(D, M, W, dp.nslots + 2);
     const int64_t total = in_list ? (int64_t)*in_count : pl.P;
     if ((int64_t)blockIdx.x * kP >= total) return;  // the whole CTA: no plan
     uint2 *ring = (uint2 *)(sm + L.ring);
+    uint16_t *next = (uint16_t *)(sm + L.next);  // [buffer][position][plan] (by next use)
     const int32_t chunks = (N + kChunk - 1) / kChunk;
     volatile uint32_t *gave_up = (volatile uint32_t *)(sm + L.flag);
 
     int32_t *weight = (int32_t *)(sm + L.weight);
-    int32_t *cap = (int32_t *)(sm + L.cap);
     int32_t *load = (int32_t *)(sm + L.load);
     uint32_t *arrival = (uint32_t *)(sm + L.arr);
     uint32_t *open = (uint32_t *)(sm + L.open);
     uint32_t *gmask = (uint32_t *)(sm + L.gmask);  // [buffer][device group][plan]
     if (threadIdx.x < 16) weight[threadIdx.x] = (int)threadIdx.x < M ? __ldg(dp.weight + threadIdx.x) : 0;
-    for (int32_t k = threadIdx.x; k < D; k += blockDim.x) cap[k] = __ldg(dp.cap + k);
     for (int32_t k = threadIdx.x; k < M * D; k += blockDim.x) load[k] = __ldg(dp.load + k);
+    if (kReclaim) {
+        for (uint32_t k = threadIdx.x; k < 64u * sizeof(Q); k += blockDim.x) {
+            uint32_t w = 0;
+            for (int32_t m = 0; m < 8; ++m)
+                if ((k >> m) & 1u) w += 8 * (int32_t)(k >> 8) + m < M ? (uint32_t)__ldg(dp.weight + 8 * (k >> 8) + m) : 0u;
+            ((uint32_t *)(sm + L.wsum))[k] = w;
+        }
+        for (int32_t k = threadIdx.x; k < M * D; k += blockDim.x)
+            ((float *)(sm + L.rcost))[k] = 1.0f / (float)max(__ldg(dp.load + k), 1);
+    }
     for (int32_t k = threadIdx.x; k < W; k += blockDim.x) arrival[k] = (uint32_t)__ldg(dp.arrival + k);
     // (each role's first __syncthreads below publishes these tables)
 
@@ -426,15 +448,14 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 h1[j] = okq[j] && i + kChunk < N && !quit ? __ldg(rp[j].order + i + kChunk) : 0;
                 act[j] = okq[j] && i < N && !quit;
                 if (kReclaim && qq[j] >= 0)  // the next use of this unit's model on its device
-                    rb[(3 * kChunk + pos) * kPitch + qq[j]] =
-                        make_uint2(act[j] ? (uint32_t)__ldg(dp.nextuse + qplan[j] * (int64_t)N + i) : 0xFFFFu, 0u);
+                    next[(b * kChunk + pos) * kPitch + qq[j]] = act[j] ? __ldg(dp.nextuse + qplan[j] * (int64_t)N + i) : (uint16_t)0xFFFFu;
             }
             uint32_t dev[kIters];
             produce_batch<kIters, kPitch>(dp, pl, rp, act, h0, rb, pos, qq, dev, open);
             // For each residency lane, the chunk's units on its devices: one
             // ballot per device group; each half-warp holds one plan.
 #pragma unroll
-            for (int j = 0; j < kIters; ++j) {
+            for (int j = 0; j < kIters && !kReclaim; ++j) {
                 const uint32_t key = dev[j] == 0xFFFFFFFFu ? (uint32_t)kG : dev[j] % kG;
 #pragma unroll
                 for (int gg = 0; gg < kG; ++gg) {
@@ -452,34 +473,24 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
             if (c >= kBuffers) named_sync(kEmpty + c % kBuffers, kProdThreads + 32);
     } else if (warp >= 1) {
         // ---------------- residency (Eq. 11, Section 3.5) ----------------
-        // Lane (plan, device group): kG lanes per plan, and lane g plays the
-        // plan's units on the devices d = g (mod kG) in dispatch order;
-        // under least-recently-used reclamation devices do not interact.
-        // Reclamation by next use counts a model's copies over all devices,
-        // so there one lane per plan plays every device.  The producers
-        // leave each lane's units of the chunk as a mask (gmask).
         const int rl = (warp - 1) * 32 + lane;
+        constexpr int kRow = PcGroups<kP, kReclaim, Q>::kLanes;
+        if constexpr (!kReclaim) {
+        // Lane (plan, device group): kG lanes per plan, and lane g plays the
+        // plan's units on the devices d = g (mod kG) in dispatch order:
+        // under least-recently-used reclamation devices do not interact.  The
+        // producers leave each lane's units of the chunk as a mask (gmask).
         const int qp = rl / kG, g = rl % kG;
         const bool rmine = qp < kP;
         const int64_t p = (rmine && qp < ng) ? (in_list ? (int64_t)in_list[j0 + qp] : j0 + qp) : 0;
         const bool live = rmine && qp < ng && out.status[p] == 0;
-        constexpr int kRow = PcGroups<kP, kReclaim>::kLanes;
-        uint32_t *used = (uint32_t *)(sm + L.used) + rl;  // [device / kG][lane] (reclamation by next use)
-        Q *queue = (Q *)(sm + L.queue) + rl;
-        uint8_t *nres = sm + L.nres + rl;
-        DevState<Q> *state = (DevState<Q> *)(sm + L.queue) + rl;  // [device / kG][lane] (least recently used)
-        uint16_t *nuse = (uint16_t *)(sm + L.nuse) + qp;  // [device][model][plan]
-        uint8_t *rcnt = sm + L.rcnt + qp;                 // [model][plan]
-        uint16_t *everl = (uint16_t *)(sm + L.everl) + rl;  // [device / kG][lane], bit m: m was held (kPhi)
-        if (rmine) {
+        DevState<Q> *state = (DevState<Q> *)(sm + L.queue) + rl;  // [device / kG][lane]
+        uint16_t *everl = (uint16_t *)(sm + L.everl) + rl;        // [device / kG][lane], bit m: m was held (kPhi)
+        if (rmine)
             for (int32_t t = 0; t * kG + g < D; ++t) {
-                if (kReclaim) { used[t * kRow] = 0; queue[t * kRow] = 0; nres[t * kRow] = 0; }
-                else state[t * kRow].init((uint32_t)__ldg(dp.cap + t * kG + g));
+                state[t * kRow].init((uint32_t)__ldg(dp.cap + t * kG + g));
                 if (kPhi) everl[t * kRow] = 0;
             }
-            if (kReclaim)
-                for (int32_t k = 0; k < M; ++k) rcnt[k * kP] = 0;
-        }
         __syncthreads();
         for (int32_t c = 0; c < chunks; ++c) {
             const int b = c % kBuffers;
@@ -495,96 +506,17 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 const int32_t kn = todo ? __ffs((int)todo) - 1 : k;
                 const uint2 nv = rb[(1 * kChunk + kn) * kPitch];
                 const uint32_t r1 = v.x, r3 = v.y;
-                const int32_t d = (int32_t)(r3 & 31u);
-                if (!kReclaim) {
-                    const int32_t t = d / kG;
-                    DevState<Q> ds = state[t * kRow];
-                    bool missed;
-                    uint2 w = ds.settle(r1, r3, weight, load, D, dp.err, missed);
-                    if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
-                        const uint32_t m = (r3 >> 5) & 15u, e = everl[t * kRow];
-                        w.x |= ((e >> m) & 1u) << 31;
-                        everl[t * kRow] = (uint16_t)(e | (1u << m));
-                    }
-                    state[t * kRow] = ds;
-                    rb[(1 * kChunk + k) * kPitch] = w;
-                } else {
-                    // Reclamation by next use: victims one at a time, a copy
-                    // also resident elsewhere first, then the largest (next
-                    // use - position) / reload cost (no next use or a free
-                    // reload: infinite), then the least recently used.
-                    const uint32_t m = (r3 >> 5) & 15u;
-                    Q q = queue[d * kRow];
-                    uint32_t n = nres[d * kRow];
-                    uint32_t u_d = used[d * kRow];  // used + need <= cap + peak < 2^32
-                    const uint32_t wm = (uint32_t)weight[m];
-                    const uint32_t capd = (uint32_t)cap[d];
-                    const bool was_empty = n == 0;
-                    const int32_t kq = Lru<Q>::find(q, n, m);
-                    const bool hit = kq < (int32_t)n;
-                    q = hit ? Lru<Q>::remove(q, hit ? kq : 0) : q;  // (an index below the queue length)
-                    n -= hit ? 1u : 0u;
-                    const uint32_t need = hit ? r1 : wm + r1;
-                    const int32_t here = c * kChunk + k;
-                    while (u_d + need > capd && n > 0) {
-                        // The class (redundant << 1 | infinite) ranks first; within
-                        // a finite class the larger distance per unit of cost
-                        // (32-bit factors, exact 64-bit products); ties keep the
-                        // earlier queue entry.
-                        int32_t best = 0;
-                        uint32_t bcls = 0;
-                        int32_t bdist = 0, bcost = 0;
-                        // (Unrolled over the queue's capacity, so the entries'
-                        // loads are not chained through the loop counter.)
-#pragma unroll
-                        for (int32_t e = 0; e < Lru<Q>::kSlots; ++e) {
-                            if (e >= (int32_t)n) break;
-                            const uint32_t kk = (uint32_t)(q >> (4 * e)) & 15u;
-                            const uint32_t red = rcnt[kk * kP] > 1;
-                            const uint32_t nu = nuse[(d * M + kk) * kP];
-                            const int32_t cost = load[kk * D + d];
-                            const uint32_t inf = nu == 0xFFFFu || cost == 0;
-                            const uint32_t cls = (red << 1) | inf;
-                            const int32_t dist = (int32_t)nu - here;
-                            if (e == 0 || cls > bcls ||
-                                (cls == bcls && !inf && (int64_t)dist * bcost > (int64_t)bdist * cost)) {
-                                best = e; bcls = cls; bdist = dist; bcost = cost;
-                            }
-                        }
-                        const uint32_t victim = (uint32_t)(q >> (4 * best)) & 15u;
-                        u_d -= (uint32_t)weight[victim];
-                        rcnt[victim * kP] -= 1;
-                        q = Lru<Q>::remove(q, best);
-                        n -= 1;
-                    }
-                    if (u_d + need > capd) atomicExch(dp.err, 2);  // unreachable for a valid plan
-                    if (!hit) rcnt[m * kP] += 1;
-                    nuse[(d * M + m) * kP] = (uint16_t)rb[(3 * kChunk + k) * kPitch].x;
-                    q |= (Q)m << (4 * n);  // the unit's model is now the most recently used
-                    n += 1;
-                    u_d += hit ? 0u : wm;
-                    uint32_t emptied = 0;
-                    if ((r3 >> 10) & 1u) {  // retain bit 0: reclaim at the end of the unit
-                        q &= ~((Q)0xF << (4 * (n - 1)));
-                        n -= 1;
-                        u_d -= wm;
-                        emptied = n == 0;
-                        rcnt[m * kP] -= 1;
-                    }
-                    queue[d * kRow] = q;
-                    nres[d * kRow] = (uint8_t)n;
-                    used[d * kRow] = u_d;
-                    uint32_t reload = 0;
-                    if (kPhi && !hit) {
-                        const uint32_t e = everl[d * kRow];
-                        reload = ((e >> m) & 1u) << 31;
-                        everl[d * kRow] = (uint16_t)(e | (1u << m));
-                    }
-                    rb[(1 * kChunk + k) * kPitch] =
-                        make_uint2(hit ? 0u : ((uint32_t)load[m * D + d] | reload),
-                                   (r3 & ~(kPrefetch | kWasEmpty)) | (hit ? 0u : (r3 & kPrefetch)) |
-                                       (was_empty ? kWasEmpty : 0u) | (emptied ? kEmptied : 0u));
+                const int32_t t = (int32_t)(r3 & 31u) / kG;
+                DevState<Q> ds = state[t * kRow];
+                bool missed;
+                uint2 w = ds.settle(r1, r3, weight, load, D, dp.err, missed);
+                if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
+                    const uint32_t m = (r3 >> 5) & 15u, e = everl[t * kRow];
+                    w.x |= ((e >> m) & 1u) << 31;
+                    everl[t * kRow] = (uint16_t)(e | (1u << m));
                 }
+                state[t * kRow] = ds;
+                rb[(1 * kChunk + k) * kPitch] = w;
                 k = kn;
                 v = nv;
             }
@@ -592,8 +524,202 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         }
         if (live) {  // devices still occupied at the end
             uint32_t o = 0;
-            for (int32_t t = 0; t * kG + g < D; ++t) o += kReclaim ? nres[t * kRow] != 0 : state[t * kRow].occupied();
+            for (int32_t t = 0; t * kG + g < D; ++t) o += state[t * kRow].occupied();
             if (o) atomicAdd(open + qp, o);
+        }
+        } else {
+        // Reclamation by next use counts a model's copies over all devices, so
+        // a plan's units are played one after another, by kL lanes that each
+        // stand for two models (l and l + kL): a lane keeps the number of each
+        // one's copies and, in shared memory, per device the copy's next use
+        // and its last use (0: not resident).  Victims go one at a time: a copy
+        // also resident elsewhere first, then the largest (next use -
+        // position) / reload cost (no next use or a free reload: infinite),
+        // then the least recently used.  None of that changes while one
+        // admission evicts, so a lane ranks its copies among the others' at
+        // once, by a float quotient, and a copy goes if those before it do
+        // not make room enough; where the float cannot tell two quotients
+        // apart (its error is below 2^-21) exact products decide.  The stage
+        // is bound by issue (about 200 instructions a unit of four plans).
+        // 16,384 plans of N = 2,000, D = M = 8, us a step: a lane per plan, which
+        // scanned the queue for each victim, 4,095; a lane per model 2,722; two
+        // models a lane (270 instructions for eight plans, half the warps) 3,010;
+        // a lane per model with a loop that takes one victim at a time 3,172.
+        constexpr int kL = kModelLanes<Q>;
+        constexpr int kI = kPer<Q>;
+        constexpr uint32_t kAll = (1u << kL) - 1u;
+        constexpr uint32_t kNear = 8;  // units in the last place: two quotients' errors are below 6
+        const int qp = rl / kL, ml = rl % kL, shift = lane & ~(kL - 1);
+        const bool rmine = qp < kP;
+        const int64_t p = (rmine && qp < ng) ? (in_list ? (int64_t)in_list[j0 + qp] : j0 + qp) : 0;
+        const bool live = rmine && qp < ng && out.status[p] == 0;
+        uint32_t *tab = (uint32_t *)(sm + L.queue) + kI * rl;           // [device][lane][l, l + kL]: next use | last use + 1 << 16
+        uint32_t *room = (uint32_t *)(sm + L.free) + (rmine ? qp : 0);  // [device][plan]: free capacity
+        const float *rcost = (const float *)(sm + L.rcost);             // [model][device]: 1 / load time
+        const uint32_t *wsum = (const uint32_t *)(sm + L.wsum);         // the weight of each set of eight models
+        int mrow[kI];
+#pragma unroll
+        for (int i = 0; i < kI; ++i) mrow[i] = (ml + i * kL < M ? ml + i * kL : 0) * D;
+        auto row_of = [&](uint32_t d, uint32_t (&x)[kI]) {
+            if constexpr (kI == 2) {
+                const uint2 u = *(const uint2 *)(tab + 2 * d * kRow);
+                x[0] = u.x; x[1] = u.y;
+            } else {
+                x[0] = tab[d * kRow];
+            }
+        };
+        auto set_row = [&](uint32_t d, const uint32_t (&x)[kI]) {
+            if constexpr (kI == 2) *(uint2 *)(tab + 2 * d * kRow) = make_uint2(x[0], x[1]);
+            else tab[d * kRow] = x[0];
+        };
+        const uint32_t none[kI] = {};
+        for (int32_t d = 0; d < D; ++d) {
+            set_row(d, none);
+            if (rmine && ml == 0) room[d * kP] = (uint32_t)__ldg(dp.cap + d);
+        }
+        __syncthreads();
+        uint32_t wx[kL][kI];  // the models' weights, of lane l ^ o
+#pragma unroll
+        for (int o = 0; o < kL; ++o)
+#pragma unroll
+            for (int i = 0; i < kI; ++i) wx[o][i] = (uint32_t)weight[(ml ^ o) + i * kL];
+        uint32_t copies[kI] = {}, ever[kI] = {};  // of the lane's models; ever: the devices that held it (kPhi)
+        for (int32_t c = 0; c < chunks; ++c) {
+            const int b = c % kBuffers;
+            named_sync(kFullP + b, kProdThreads + kResThreads);
+            uint2 *rb = ring + b * kRW * kChunk * kPitch + (rmine ? qp : 0);
+            const uint16_t *nb = next + b * kChunk * kPitch + (rmine ? qp : 0);
+            const int32_t kmax = min(kChunk, N - c * kChunk);
+            uint2 v = rb[1 * kChunk * kPitch];
+            uint32_t nu = nb[0];
+#pragma unroll 1
+            for (int32_t k = 0; k < kmax; ++k) {
+                const int32_t kn = min(k + 1, kChunk - 1);
+                const uint2 nv = rb[(1 * kChunk + kn) * kPitch];
+                const uint32_t nnu = nb[kn * kPitch];
+                const bool act = live && !(v.y & kSkip);
+                const uint32_t r1 = v.x, r3 = act ? v.y : 0u, m = (r3 >> 5) & 15u, d = r3 & 31u;
+                uint32_t x[kI];
+                row_of(d, x);
+                uint32_t f = room[d * kP];
+                const uint32_t wm = (uint32_t)weight[m], ld = (uint32_t)load[m * D + d];
+                const int32_t here = c * kChunk + k;
+                uint32_t held = 0;  // the models on the device
+#pragma unroll
+                for (int i = 0; i < kI; ++i) held |= ((__ballot_sync(0xFFFFFFFFu, x[i] >> 16) >> shift) & kAll) << (i * kL);
+                const bool was_empty = held == 0, hit = (held >> m) & 1u;
+                held &= ~(1u << m);
+                const uint32_t need = hit ? r1 : wm + r1;  // at most the capacity
+                if (__any_sync(0xFFFFFFFFu, act && need > f)) {
+                    int32_t cost[kI], dist[kI];  // cost 0 (and distance 1): infinite
+                    uint32_t key[kI], ahead[kI], nearest[kI];
+#pragma unroll
+                    for (int i = 0; i < kI; ++i) {
+                        cost[i] = load[mrow[i] + d];
+                        const uint32_t nuse = x[i] & 0xFFFFu;
+                        const bool inf = nuse == 0xFFFFu || cost[i] == 0;
+                        dist[i] = inf ? 1 : (int32_t)nuse - here;
+                        // (infinite: in the order of last use, and too far apart to be called near)
+                        const uint32_t q = inf ? 0x7F800000u + ((0xFFFFu - (x[i] >> 16)) << 4)
+                                               : __float_as_uint((float)dist[i] * rcost[mrow[i] + d]);
+                        key[i] = (held >> (ml + i * kL)) & 1u ? (copies[i] > 1 ? 0x80000000u : 0u) | q : 0u;
+                        cost[i] = inf ? 0 : cost[i];
+                    }
+                    // The weight of the copies that go before each of this lane's, and how near the nearest quotient is.
+                    if constexpr (kI == 2) {
+                        ahead[0] = key[1] > key[0] ? wx[0][1] : 0u;
+                        ahead[1] = key[0] > key[1] ? wx[0][0] : 0u;
+                        nearest[0] = key[1] - key[0] + kNear;
+                        nearest[1] = key[0] - key[1] + kNear;
+                    } else {
+                        ahead[0] = 0;
+                        nearest[0] = ~0u;
+                    }
+#pragma unroll
+                    for (int o = 1; o < kL; ++o)
+#pragma unroll
+                        for (int j = 0; j < kI; ++j) {
+                            const uint32_t pk = __shfl_xor_sync(0xFFFFFFFFu, key[j], o);
+#pragma unroll
+                            for (int i = 0; i < kI; ++i) {
+                                if (pk > key[i]) ahead[i] += wx[o][j];
+                                nearest[i] = min(nearest[i], pk - key[i] + kNear);
+                            }
+                        }
+                    bool close = false;
+#pragma unroll
+                    for (int i = 0; i < kI; ++i) close |= key[i] && nearest[i] <= 2 * kNear;
+                    if (__any_sync(0xFFFFFFFFu, close && act && need > f)) {
+#pragma unroll
+                        for (int i = 0; i < kI; ++i) ahead[i] = 0;
+                        for (int o = 0; o < kL; ++o)
+#pragma unroll
+                            for (int j = 0; j < kI; ++j) {
+                                const uint32_t pk = __shfl_xor_sync(0xFFFFFFFFu, key[j], o), ps = __shfl_xor_sync(0xFFFFFFFFu, x[j] >> 16, o);
+                                const int32_t pd = __shfl_xor_sync(0xFFFFFFFFu, dist[j], o), pc = __shfl_xor_sync(0xFFFFFFFFu, cost[j], o);
+#pragma unroll
+                                for (int i = 0; i < kI; ++i) {
+                                    bool before = pk > key[i];
+                                    if (key[i] && pk - key[i] + kNear <= 2 * kNear) {
+                                        const int64_t l = (int64_t)pd * cost[i], r = (int64_t)dist[i] * pc;
+                                        before = l > r || (l == r && ps < x[i] >> 16);  // (never before itself)
+                                    }
+                                    if (before) ahead[i] += (uint32_t)weight[(ml ^ o) + j * kL];
+                                }
+                            }
+                    }
+                    uint32_t gone = 0;
+#pragma unroll
+                    for (int i = 0; i < kI; ++i) {
+                        const bool goes = act && key[i] && need > f + ahead[i];
+                        gone |= ((__ballot_sync(0xFFFFFFFFu, goes) >> shift) & kAll) << (i * kL);
+                        if (goes) { x[i] = 0; copies[i] -= 1; }
+                    }
+                    held &= ~gone;
+                    f += wsum[gone & 255u];
+                    if (sizeof(Q) > 4) f += wsum[256 + (gone >> 8)];
+                    if (act && need > f) atomicExch(dp.err, 2);  // unreachable for a valid plan
+                }
+                const bool drop = (r3 & kDrop) != 0;  // the model leaves when the unit ends
+                if (!hit && !drop) f -= wm;
+                if (hit && drop) f += wm;
+                if (act) {
+                    const uint32_t mine = drop ? 0u : nu | ((uint32_t)(here + 1) << 16);
+                    const uint32_t more = (hit ? 0u : 1u) - (drop ? 1u : 0u);
+                    uint32_t reload = 0;
+#pragma unroll
+                    for (int i = 0; i < kI; ++i)
+                        if ((uint32_t)(ml + i * kL) == m) {
+                            copies[i] += more;
+                            x[i] = mine;
+                            if (kPhi && !hit) {
+                                reload = ((ever[i] >> d) & 1u) << 31;
+                                ever[i] |= 1u << d;
+                            }
+                        }
+                    if ((uint32_t)ml == m % kL) {
+                        uint2 w = settled(r3, hit, ld, was_empty, drop && held == 0);
+                        if (kPhi) w.x |= reload;
+                        room[d * kP] = f;
+                        rb[(1 * kChunk + k) * kPitch] = w;
+                    }
+                    set_row(d, x);
+                }
+                __syncwarp();  // the free capacity is written
+                v = nv;
+                nu = nnu;
+            }
+            named_arrive(kFullR + b, kResThreads + 32);
+        }
+        uint32_t o = 0;  // devices still occupied at the end
+        for (int32_t d = 0; d < D; ++d) {
+            uint32_t x[kI], any = 0;
+            row_of(d, x);
+#pragma unroll
+            for (int i = 0; i < kI; ++i) any |= x[i] >> 16;
+            o += ((__ballot_sync(0xFFFFFFFFu, any) >> shift) & kAll) != 0;
+        }
+        if (live && ml == 0 && o) atomicAdd(open + qp, o);
         }
         named_arrive(kOpen, kResThreads + 32);
     } else {
@@ -838,18 +964,32 @@ nextuse_kernel(wf_dev_problem dp, wf_plans pl, const uint32_t *status, uint16_t 
         uint16_t *out = table + p * (int64_t)N;
         for (int32_t k = lane; k < D * M; k += 32) last[k] = 0xFFFFu;
         __syncwarp();
+        // Three chunks of gathers are in flight ahead of the one being settled:
+        // its dispatch entries, then their nodes' placement, record and fusion
+        // word, then the placement of their fusible predecessors.
+        const int32_t top = ((N - 1) / 32) * 32 + lane;
+        auto entry = [&](int32_t j) { return j >= 0 && j < N ? (int32_t)__ldg(order + j) : 0; };
+        struct Node {
+            uint32_t d, x, links, model, fw;
+        };
+        auto node = [&](int32_t h) {
+            const uint4 hr = __ldg(dp.hrec + h);
+            return Node{__ldg(place + h), (uint32_t)h, hr.x, (hr.y >> 16) & 15u, __ldg(fuse + (h >> 5))};
+        };
+        auto before = [&](const Node &n) { return (n.links & 0xFFFFu) != 0xFFFFu ? (uint32_t)__ldg(place + (n.links & 0xFFFFu)) : ~0u; };
+        Node n1 = node(entry(top)), n2 = node(entry(top - 32));
+        uint32_t p1 = before(n1);
+        int32_t h3 = entry(top - 64);
         for (int32_t base = ((N - 1) / 32) * 32; base >= 0; base -= 32) {
             const int32_t j = base + lane;
+            const Node n = n1;
+            const uint32_t pn = p1;
+            n1 = n2;
+            p1 = before(n1);
+            n2 = node(h3);
+            h3 = entry(j - 96);
             uint32_t key = 0xFFFFFFFFu;  // not the start of a unit
-            if (j < N) {
-                const int32_t x = __ldg(order + j);
-                const int32_t d = __ldg(place + x);
-                const uint4 hr = __ldg(dp.hrec + x);
-                const uint32_t fp = hr.x & 0xFFFFu;
-                const bool member = fp != 0xFFFFu && ((__ldg(fuse + (x >> 5)) >> (x & 31)) & 1u) &&
-                                    __ldg(place + fp) == d;
-                if (!member) key = (uint32_t)d * M + ((hr.y >> 16) & 15u);
-            }
+            if (j < N && !(((n.fw >> (n.x & 31)) & 1u) && pn == n.d)) key = n.d * M + n.model;
             const uint32_t same = __match_any_sync(0xFFFFFFFFu, key);
             const uint32_t above = lane == 31 ? 0u : (same & (0xFFFFFFFFu << (lane + 1)));
             if (key != 0xFFFFFFFFu) out[j] = above ? (uint16_t)(base + __ffs((int)above) - 1) : last[key];
@@ -1081,7 +1221,7 @@ int launch_pc(const wf_dev_problem &dp, int sms, int resident, const wf_plans *p
     // many CTAs as are resident at once, each walking over groups.
     int64_t blocks = (pl->P + kP - 1) / kP;
     if (in_list) blocks = std::min<int64_t>(blocks, (int64_t)std::max(1, resident) * sms);
-    pc_kernel<Q, TT, kP, kR, kF, ST><<<(unsigned)blocks, 32 * PcShape<kP>::kWarps, smem, st>>>(
+    pc_kernel<Q, TT, kP, kR, kF, ST><<<(unsigned)blocks, 32 * PcShape<kP, kR, Q>::kWarps, smem, st>>>(
         dp, *pl, *out, in_list, in_count, list, count);
     return wf_cuda_check(cudaGetLastError(), "sweep launch");
 }
@@ -1098,6 +1238,8 @@ int pc_visit(const wf_dev_problem &dp, int kp, F &&f)
     } else {
         auto by_q = [&](auto p, auto s) { return dp.M <= 8 ? f(Ty<uint32_t>{}, p, s) : f(Ty<uint64_t>{}, p, s); };
         auto by_p = [&](auto s) {
+            if constexpr (kR != 0)
+                if (kp == 2) return by_q(Iv<2>{}, s);
             return kp == 16 ? by_q(Iv<16>{}, s) : kp == 6 ? by_q(Iv<6>{}, s) : by_q(Iv<3>{}, s);
         };
         if constexpr (kR == 0)
@@ -1127,8 +1269,8 @@ int resident_r(const wf_dev_problem &dp, int kp, size_t smem)
         const auto k = pc_kernel<typename decltype(q)::type, TT, decltype(p)::value, kR, kF, typename decltype(s)::type>;
         int n = 0;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, 32 * PcShape<decltype(p)::value>::kWarps, smem) !=
-                cudaSuccess) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &n, k, 32 * PcShape<decltype(p)::value, kR, typename decltype(q)::type>::kWarps, smem) != cudaSuccess) {
             (void)cudaGetLastError();
             return 0;
         }
@@ -1253,6 +1395,19 @@ struct CfgKey {
     }
 };
 
+// The windows that take reclamation by next use: those of which three plans
+// fit a CTA with a lane's state per plan and device (16-bit next uses, a queue
+// word).  The state per model is up to 8 KB larger, so near that limit the
+// 64-bit sweep plays two plans a CTA.
+bool next_use_window(const wf_dev_problem &dp)
+{
+    const int32_t D = dp.D, M = dp.M;
+    const size_t o = 64 + round16(4u * D) + round16(4u * M * D) + round16(4u * dp.W) + 4608 + round16(24u * (dp.nslots + 2)) +
+                     round16(24u * D) + round16((M <= 8 ? 12u : 24u) * D) + round16(12u * D) + round16(3u * D) + 32 +
+                     round16(6u * D * M) + round16(3u * M) + 48 + (dp.phi_life ? round16(6u * D) : 0u);
+    return o <= 227 * 1024;
+}
+
 wf_sweep_cfg choose(const wf_dev_problem &dp)
 {
     wf_sweep_cfg c = {};
@@ -1275,6 +1430,14 @@ wf_sweep_cfg choose(const wf_dev_problem &dp)
             c.smem64 = sm;
             c.plans64 = kp;
             c.res64 = n;
+        }
+    }
+    if (!c.smem64 && dp.reclaim && next_use_window(dp)) {
+        const size_t sm = layout_bytes<2, uint64_t>(dp);
+        c.res64 = resident<uint64_t>(dp, 2, sm);
+        if (c.res64 > 0) {
+            c.smem64 = sm;
+            c.plans64 = 2;
         }
     }
     // The relative-time sweep (for contexts whose plans leave 32 bits): 6 or

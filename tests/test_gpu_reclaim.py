@@ -79,3 +79,33 @@ def test_stochastic_problems_refuse_the_policy():
     ctx = wf.Ctx(w.problem, max_P=8)
     with pytest.raises(wf.WfError):
         wf.wf_ctx_set_reclaim(ctx, 1)
+
+
+@pytest.mark.parametrize("loads", ["zero", "equal", "powers", "near", "huge"])
+@pytest.mark.parametrize("D,M", [(3, 7), (6, 8), (32, 9), (5, 16)])
+def test_tied_and_nearly_tied_quotients(loads, D, M):
+    """Reload costs whose quotients tie exactly (all equal, powers of two), come
+    within a few units in the last place of a float (2^24 + a little, and up
+    to 2^31 - 1), or are infinite (no reload cost)."""
+    rng = np.random.default_rng(3200 + 10 * D + M)
+    prob = random_problem(rng, n_sessions=9, sizes=(8, 16), D=D, M=M)
+    m = np.arange(M)[:, None] + np.zeros((1, D), np.int64)
+    load = {"zero": m * 0, "equal": m * 0 + 48, "powers": 1 << (m % 6), "near": (1 << 24) * (1 + m % 3) + rng.integers(0, 3, (M, D)),
+            "huge": (1 << 31) - 1 - rng.integers(0, 4, (M, D)) * (1 + m % 2)}[loads]
+    prob = prob.with_(reclaim=1, load_us=load.reshape(-1).astype(np.int32))
+    plans = wfgen.make_plans(prob, 200, D + M, p_retain=0.7 if D % 2 else None)
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
+
+
+def test_largest_window():
+    """A window near the shared-memory limit of the policy (32 devices, 16
+    models, 7,800 sessions), where the sweep plays two plans per CTA."""
+    rng = np.random.default_rng(3300)
+    W, D, M = 7800, 32, 16
+    dev = wfgen.DeviceSpec(cap_gib=[60 + d for d in range(D)], speed=[1.0] * D, bw_gbps=[1] * D)
+    prob = wfgen.assemble("wide", [[("planner", [])] for _ in range(W)], np.sort(rng.integers(0, 500, W)).astype(np.int64), dev,
+                          [5 + m for m in range(M)], rng, lat_median_us=100, lat_sigma=0.6, kv_lo=1, kv_hi=20)
+    prob = prob.with_(reclaim=1, model=rng.integers(0, M, W).astype(prob.model.dtype))
+    prob = prob.with_(peak_mib=np.repeat(prob.weight_mib[prob.model] + 64, D).astype(np.int32))
+    plans = wfgen.make_plans(prob, 5, 1)
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
