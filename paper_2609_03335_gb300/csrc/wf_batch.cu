@@ -330,11 +330,11 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 publish<TT>(slots, r3 >> 16, cfin);  // the sink when the unit writes nothing
                 publish<TT>(slots, r4 & 0xFFFFu, cfin);
                 const uint32_t nwl = (r3 >> 11) & 7u;
-                if (nwl > 2) {
+                if (r3 & kMany) {
                     publish<TT>(slots, r4 >> 16, cfin);
-                    if (nwl == 4) {
+                    if (nwl == kWrites4) {
                         publish<TT>(slots, r5 & 0xFFFFu, cfin);
-                    } else if (nwl > 4) {  // five or more codes: the list from global memory
+                    } else if (nwl > kWrites4) {  // five or more codes: the list from global memory
                         const int4 wr = __ldg(dp.noderec + 2 * (int32_t)(r5 & 0xFFFFu) + 1);
                         for (int32_t e = 3; e < wr.y; ++e) publish<TT>(slots, __ldg(dp.wl + wr.x + e), cfin);
                     }

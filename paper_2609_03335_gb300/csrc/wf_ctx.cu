@@ -258,7 +258,7 @@ extern "C" int wf_ctx_create(const wf_problem *pb, int device, int64_t max_P, wf
     size_t o_links = img.add(links.data(), sizeof(uint32_t) * N);
     // Per-node record of the sweep's producers: links; release slot code
     // (slot | accumulator << 15; the zero slot nslots + 1 without
-    // predecessors) | model << 16 | write-list length (max 7) << 20; session
+    // predecessors) | model << 16 | writes field (0, 4, 5 or 6) << 20; session
     // arrival (u32: the sweep runs only with arrivals below 2^32); the first
     // two write codes, the sink slot nslots standing in for absent ones.
     std::vector<uint4> hrec(N);
@@ -270,7 +270,7 @@ extern "C" int wf_ctx_create(const wf_problem *pb, int device, int64_t max_P, wf
                                              : (((uint32_t)rslot[n] & 0x7FFFu) | ((rslot[n] & WF_RSLOT_ACC) ? 0x8000u : 0u));
             const int32_t a = wl_off[n], len = wl_off[n + 1] - wl_off[n];
             const uint32_t c0 = len > 0 ? wl[a] : trash, c1 = len > 1 ? wl[a + 1] : trash;
-            hrec[n] = make_uint4(links[n], rs | ((uint32_t)pb->model[n] << 16) | ((uint32_t)std::min(len, 7) << 20),
+            hrec[n] = make_uint4(links[n], rs | ((uint32_t)pb->model[n] << 16) | ((len <= 2 ? 0u : (uint32_t)std::min(len, 5) + 1u) << 20),
                                  (uint32_t)pb->arrival_us[pb->session[n]], c0 | (c1 << 16));
             wc23[n] = (len > 2 ? wl[a + 2] : trash) | ((uint32_t)(len > 3 ? wl[a + 3] : trash) << 16);
         }

@@ -88,6 +88,10 @@ constexpr uint32_t kDrop = 1u << 10;       // before residency: the unit's model
 constexpr uint32_t kWasEmpty = 1u << 10;   // after residency: a miss on an empty device
 constexpr uint32_t kEmptied = 1u << 15;    // after residency: the unit's reclaim empties the device
 constexpr uint32_t kRunCap = 0xFFFFFFFFu;  // saturation of w0
+// The writes field: 0 for up to two codes (which every record holds), 4 for
+// three, 5 for four, 6 for more; kMany tests for more than two.
+constexpr uint32_t kMany = 1u << 13;
+constexpr uint32_t kWrites4 = 5;
 // A plan's open word in shared memory: the devices still occupied at its end
 // (residency, low bits) and, from bit kOpenBad, the placement status bits
 // (WF_ST_DEVICE, WF_ST_CAPACITY) its producers found.
@@ -289,6 +293,16 @@ __device__ __forceinline__ void l2_prefetch(const void *p, uint32_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// A record that starts no unit, which the timing stages may also play: no run
+// time, no load, device 0, the zero slot read and the sink written.
+template <int kPitch>
+__device__ __forceinline__ void skip_record(uint2 *dst, uint32_t sink)
+{
+    dst[0] = make_uint2(0u, 0u);
+    dst[1 * kChunk * kPitch] = make_uint2(0u, kSkip | (sink << 16));
+    dst[2 * kChunk * kPitch] = make_uint2(sink | (sink << 16), (sink + 1) << 16);
+}
+
 // The records of kI (plan, position) pairs at once, with the gathers of all
 // pairs issued together in three dependent rounds: the head's own tables
 // (placement, node record, fusion / prefetch / retain words, third and
@@ -344,9 +358,7 @@ __device__ __forceinline__ void produce_batch(const wf_dev_problem &dp, const wf
         if (act[j] && !bad[j] && lk0[j].y < 0) bad[j] = (uint32_t)WF_ST_CAPACITY;  // (d was cleared for a bad device)
         if (bad[j]) atomicOr(open + qq[j], bad[j] << kOpenBad);
         if (!act[j] || bad[j] || (((fw[j] >> (h & 31)) & 1u) && pprev[j] == d[j])) {  // no unit, or inside its head's
-            dst[0] = make_uint2(0u, 0u);
-            dst[1 * kChunk * kPitch] = make_uint2(0u, kSkip);
-            dst[2 * kChunk * kPitch] = make_uint2(0u, 0u);
+            skip_record<kPitch>(dst, (uint32_t)dp.nslots);
             continue;
         }
         uint32_t run = (uint32_t)lk0[j].x + (uint32_t)dp.grant, ovf = 0;  // both < 2^31: no wrap
@@ -374,21 +386,30 @@ __device__ __forceinline__ void produce_batch(const wf_dev_problem &dp, const wf
         }
         if (cbad) {  // (the member's own position flags the plan as well)
             atomicOr(open + qq[j], (uint32_t)WF_ST_CAPACITY << kOpenBad);
-            dst[0] = make_uint2(0u, 0u);
-            dst[1 * kChunk * kPitch] = make_uint2(0u, kSkip);
-            dst[2 * kChunk * kPitch] = make_uint2(0u, 0u);
+            skip_record<kPitch>(dst, (uint32_t)dp.nslots);
             continue;
         }
-        const uint32_t nwl = (ty >> 20) & 7u;
+        const uint32_t nwl = (ty >> 20) & 7u, rs = hr[j].y & 0xFFFFu;
+        // A code naming the accumulator that this unit reads and resets finds 0 there: a plain write.
+        if ((tw & 0xFFFFu) == rs) tw &= 0xFFFF7FFFu;
+        if ((tw >> 16) == rs) tw &= 0x7FFFFFFFu;
         const uint32_t pf = (pw[j] >> (h & 31)) & 1u;
         const uint32_t reclaim = ((rwt >> (tail & 31)) & 1u) ^ 1u;
         dst[0] = make_uint2(ovf ? kRunCap : run, hr[j].z);
         dst[1 * kChunk * kPitch] = make_uint2(
             (uint32_t)kv, d[j] | (((hr[j].y >> 16) & 15u) << 5) | (pf << 9) | (reclaim << 10) | (nwl << 11) | (tw << 16));
         dst[2 * kChunk * kPitch] = make_uint2((tw >> 16) | (c2t << 16),
-                                              (nwl == 4 ? c2t >> 16 : (uint32_t)tail) | (hr[j].y << 16));
+                                              (nwl == kWrites4 ? c2t >> 16 : (uint32_t)tail) | (hr[j].y << 16));
         dev[j] = d[j];
     }
+}
+
+// a + b on 32 bits; the carry is counted in ovf.
+__device__ __forceinline__ uint32_t add_carry(uint32_t a, uint32_t b, uint32_t &ovf)
+{
+    uint32_t c;
+    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %1, 0;" : "=r"(c), "+r"(ovf) : "r"(a), "r"(b));
+    return c;
 }
 
 // A finish time into a slot: an accumulator keeps the latest of its

@@ -88,14 +88,6 @@ __device__ __forceinline__ void put(uint32_t *p, const uint32_t (&x)[kV])
     else *p = x[0];
 }
 
-// a + b on 32 bits; the carry is counted in ovf.
-__device__ __forceinline__ uint32_t add_carry(uint32_t a, uint32_t b, uint32_t &ovf)
-{
-    uint32_t c;
-    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %1, 0;" : "=r"(c), "+r"(ovf) : "r"(a), "r"(b));
-    return c;
-}
-
 // The Box-Muller tables: radius and angle as int16 copies in shared memory
 // (kTab), or the problem's int32 tables in global memory (values beyond 16 bits, or
 // tables too long for shared memory).
@@ -239,7 +231,7 @@ stoch_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, StochShape sh, int
                 if (unit) {
                     const uint2 x = res[lane];
                     uint4 *dst = ring + 2 * (buf * kPos + __popc(units & ((1u << lane) - 1u)));
-                    const bool rare = (x.y & (kWasEmpty | kEmptied)) || ((x.y >> 11) & 7u) > 2;
+                    const bool rare = (x.y & (kWasEmpty | kEmptied)) || (x.y & kMany);
                     dst[0] = make_uint4((uint32_t)h | (tail << 16), lat, hr.z, (x.y & ~(15u << 5)) | (rare ? kRare : 0u));
                     dst[1] = make_uint4(r4, c4 | (hr.y << 16), x.x, 0u);
                 }
@@ -371,9 +363,9 @@ stoch_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, StochShape sh, int
                             put<kV>(sp, x);
                         };
                         const uint32_t nwl = (a.w >> 11) & 7u;
-                        if (nwl > 2) publish_at(b.x >> 16);
-                        if (nwl > 3) publish_at(b.y & 0xFFFFu);
-                        if (nwl > 4) {
+                        if (a.w & kMany) publish_at(b.x >> 16);
+                        if (nwl >= kWrites4) publish_at(b.y & 0xFFFFu);
+                        if (nwl > kWrites4) {
                             const int4 wr = __ldg(dp.noderec + 2 * (int32_t)(a.x >> 16) + 1);
                             for (int32_t e = 4; e < wr.y; ++e) publish_at(__ldg(dp.wl + wr.x + e));
                         }

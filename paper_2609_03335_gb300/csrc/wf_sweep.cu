@@ -77,8 +77,10 @@ struct PcShape {
     static constexpr int kRes = kReclaim ? (kP * kModelLanes<Q> + 31) / 32 : kP >= 32 ? 4 : kP >= 16 ? 2 : 1;  // residency warps
     static constexpr int kWarps = 1 + kRes + kProducers;
     // Four 16-plan CTAs share an SM (shared memory allows it at 2,000
-    // activations), which bounds the registers per thread.
-    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP < 16 ? 1 : kReclaim && sizeof(Q) == 8 ? 3 : 4;
+    // activations), or four 6-plan CTAs at 8,192, which bounds the registers
+    // per thread (large window with three of the latter, at 106 registers:
+    // 56.0 ms, with four 47.4).
+    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP < 6 ? 1 : kP < 16 ? 4 : kReclaim && sizeof(Q) == 8 ? 3 : 4;
     // Elements (8-byte word pairs) per (pair, position) row of the ring.  A
     // producer store covers 16 positions x 2 plans in two halves of 16
     // lanes; an odd pitch puts each half's 16 pairs on 32 distinct banks, and
@@ -804,46 +806,59 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
             }
         }
         const uint2 *rb = ring + b * kRW * kChunk * kPitch + lane;
-        const int32_t kmax = min(kChunk, N - c * kChunk);
         if (live) {
-            // The ring words of the next position are read while this one plays.
+            // The ring words of the next position are read while this one
+            // plays.  A skip record plays as a unit that changes nothing (no
+            // run time, no load, the zero slot, the sink), so every lane
+            // plays every position of the chunk without branching.
             uint2 w[3];
 #pragma unroll
             for (int x = 0; x < 3; ++x) w[x] = rb[(x * kChunk) * kPitch];
-            for (int32_t k = 0; k < kmax; ++k) {
-                const int32_t kn = k + 1 < kmax ? k + 1 : k;
+#pragma unroll 4
+            for (int32_t k = 0; k < kChunk; ++k) {
+                const int32_t kn = min(k + 1, kChunk - 1);
                 uint2 nw[3];
 #pragma unroll
                 for (int x = 0; x < 3; ++x) nw[x] = rb[(x * kChunk + kn) * kPitch];
                 const uint32_t r3 = w[1].y;
-                if (!(r3 & kSkip)) {
-                    const uint32_t run = w[0].x, arr = kRel ? max(w[0].y, bc) - bc : w[0].y, r4 = w[2].x,
-                                   r5 = w[2].y;
-                    const uint32_t ld = kPhi ? w[1].x & 0x7FFFFFFFu : w[1].x;  // bit 31: a reload (kPhi)
-                    TT *tf_d = tfree + (r3 & 31u) * kP;
-                    // Release (Eq. 2, Eq. 7); an accumulator slot is reset by its reader.
-                    const uint32_t rs = r5 >> 16;
-                    const TT rel = max((TT)arr, slots.get(rs & 0x7FFFu));
-                    slots.set((rs & 0x8000u) ? (rs & 0x7FFFu) : trash, 0);
-                    // A miss loads on this device first (ld > 0 only on a miss); a
-                    // prefetched load waits only for the arrival (Eq. 5).  On a hit
-                    // the residency stage cleared the prefetch bit and ld is 0.
-                    const TT tf = *tf_d;
-                    const TT ls = max(tf, (r3 & kPrefetch) ? (TT)arr : rel);
-                    const TT le = ls + ld;
-                    const TT start = max(le, rel);
-                    if (kPhi) {
-                        // A prefetched load (the bit survives residency only on a
-                        // miss) that starts before the release and ends by it is
-                        // timely; every unit adds the delay its load puts on its
-                        // start, and a reload its load time.
-                        ph_timely += (r3 & kPrefetch) && ls < rel && le <= rel;
-                        ph_life += (uint64_t)(start - max(tf, rel)) + (w[1].x >> 31 ? (uint64_t)ld : 0ull);
-                    }
-                    const TT cfin = start + run;
-                    if (kNarrow) ovf |= (le < ls) | (cfin < start);
-                    else ovf |= run == kRunCap;
-                    end = max(end, cfin);
+                const uint32_t run = w[0].x, arr = kRel ? max(w[0].y, bc) - bc : w[0].y, r4 = w[2].x, r5 = w[2].y;
+                const uint32_t ld = kPhi ? w[1].x & 0x7FFFFFFFu : w[1].x;  // bit 31: a reload (kPhi)
+                TT *tf_d = tfree + (r3 & 31u) * kP;
+                // Every slot of the unit is read before any is written (the
+                // producers took the accumulator bit off a code that names
+                // the slot which this unit resets).
+                const uint32_t rs = r5 >> 16, i0 = (r3 >> 16) & 0x7FFFu, i1 = r4 & 0x7FFFu;
+                const TT rel = max((TT)arr, slots.get(rs & 0x7FFFu));  // release (Eq. 2, Eq. 7)
+                const TT tf = *tf_d, old0 = slots.get(i0), old1 = slots.get(i1);
+                // A miss loads on this device first (ld > 0 only on a miss); a
+                // prefetched load waits only for the arrival (Eq. 5).  On a hit
+                // the residency stage cleared the prefetch bit and ld is 0.
+                const TT ls = max(tf, (r3 & kPrefetch) ? (TT)arr : rel);
+                TT le, start, cfin;
+                if constexpr (kNarrow) {
+                    le = add_carry(ls, ld, ovf);
+                    start = max(le, rel);
+                    cfin = add_carry(start, run, ovf);
+                } else {
+                    le = ls + ld;
+                    start = max(le, rel);
+                    cfin = start + run;
+                    ovf |= run == kRunCap;
+                }
+                if (kPhi) {
+                    // A prefetched load (the bit survives residency only on a
+                    // miss) that starts before the release and ends by it is
+                    // timely; every unit adds the delay its load puts on its
+                    // start, and a reload its load time.
+                    ph_timely += (r3 & kPrefetch) && ls < rel && le <= rel;
+                    ph_life += (uint64_t)(start - max(tf, rel)) + (w[1].x >> 31 ? (uint64_t)ld : 0ull);
+                }
+                end = max(end, cfin);
+                slots.set((rs & 0x8000u) ? (rs & 0x7FFFu) : trash, 0);  // an accumulator is reset by its reader
+                slots.set(i0, (r3 & 0x80000000u) ? max(old0, cfin) : cfin);  // the sink when the unit writes nothing
+                slots.set(i1, (r4 & 0x8000u) ? max(old1, cfin) : cfin);
+                *tf_d = cfin;
+                if (r3 & (kMany | kWasEmpty | kEmptied)) {
                     if (r3 & kWasEmpty) {  // an empty device becomes occupied
                         gsum -= (int64_t)ls;
                         if (kRel) --net;
@@ -852,20 +867,16 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                         gsum += (int64_t)cfin;
                         if (kRel) ++net;
                     }
-
-                    publish<TT>(slots, r3 >> 16, cfin);  // the sink when the unit writes nothing
-                    publish<TT>(slots, r4 & 0xFFFFu, cfin);
-                    const uint32_t nwl = (r3 >> 11) & 7u;
-                    if (nwl > 2) {
+                    if (r3 & kMany) {
                         publish<TT>(slots, r4 >> 16, cfin);
-                        if (nwl == 4) {
+                        const uint32_t nwl = (r3 >> 11) & 7u;
+                        if (nwl == kWrites4) {
                             publish<TT>(slots, r5 & 0xFFFFu, cfin);
-                        } else if (nwl > 4) {  // five or more codes: the list from global memory
+                        } else if (nwl > kWrites4) {  // five or more codes: the list from global memory
                             const int4 wr = __ldg(dp.noderec + 2 * (int32_t)(r5 & 0xFFFFu) + 1);
                             for (int32_t e = 3; e < wr.y; ++e) publish<TT>(slots, __ldg(dp.wl + wr.x + e), cfin);
                         }
                     }
-                    *tf_d = cfin;
                 }
 #pragma unroll
                 for (int x = 0; x < 3; ++x) w[x] = nw[x];
