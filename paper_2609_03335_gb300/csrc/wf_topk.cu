@@ -10,12 +10,18 @@
 //     tile (massive ties) are folded tile by tile into the running best k.
 //
 // Up to kOneCta plans, one CTA does all three with the keys staged in shared
-// memory (one launch): T is the exact k-th smallest key, found by radix
+// memory (one launch): T is a bound near the k-th smallest key, found by radix
 // selection (8 bits a pass, the digit found by a warp scan of the
-// histogram), so usually about k candidates reach the sort.  Beyond, T is
+// histogram) that stops once few enough keys are left.  Beyond, T is
 // first the smallest of the tiles' own k-th keys (kth_kernel, one CTA a
 // tile); the final CTA then runs the same exact selection over those
 // candidates before sorting.
+//
+// What bounds it is the chain of barriers and shared-memory passes of one
+// CTA.  Radix passes down to the exact k-th key and a sorting network took
+// 24.9 us at 16,384 plans, k = 32, and 16.3 us at 1,024 plans, k = 8; with passes
+// that end at kFew candidates or fewer, ranked by comparing each with all,
+// 16.5 and 9.0 us.
 #include <algorithm>
 
 #include "wf_internal.cuh"
@@ -23,6 +29,7 @@
 namespace {
 
 constexpr int kTile = 2048;
+constexpr int kFew = 128;  // as many candidates are ranked by comparing each with all (select_and_sort)
 constexpr int kThreads = 1024;
 
 struct Cand {
@@ -118,9 +125,10 @@ __device__ void first_pass(uint64_t mn, uint64_t mx, unsigned long long *wmin, u
 
 // The digit of the k-th smallest key in this radix pass: warp 0 scans the
 // 256-bucket histogram (8 buckets a lane), finds the bucket holding rank,
-// and narrows prefix and rank to it.
+// and narrows prefix and rank to it; after is the number of the bucket's
+// keys from that rank on.
 __device__ __forceinline__ void pick_digit(const unsigned int *hist, int shift, unsigned long long &prefix,
-                                           long long &rank)
+                                           long long &rank, long long &after)
 {
     const int lane = threadIdx.x & 31;
     unsigned int h[8], sum = 0;
@@ -138,7 +146,16 @@ __device__ __forceinline__ void pick_digit(const unsigned int *hist, int shift, 
     if (lane == src) {
         long long left = r - (long long)(inc - sum);
         int b = 0;
-        while ((long long)h[b] <= left) { left -= h[b]; ++b; }
+        unsigned int in = 0;  // the bucket's keys
+        bool found = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (found) continue;
+            in = h[j];
+            if ((long long)in > left) found = true;
+            else { left -= in; ++b; }
+        }
+        after = (long long)in - left;
         rank = left;
         prefix |= (unsigned long long)(8 * lane + b) << shift;
     }
@@ -173,15 +190,18 @@ __global__ void compact_kernel(wf_eval_out res, Terms tm, int64_t P, void *scr)
     }
 }
 
-// The k-th smallest of kk[0, n) (shared memory, k <= n), by radix selection
-// from the highest byte in which the keys differ.  Every thread of the CTA
-// calls it with the smallest and largest of the keys it wrote.
-__device__ unsigned long long radix_kth(const unsigned long long *kk, int64_t n, int32_t k, uint64_t mn,
-                                        uint64_t mx)
+// A bound that at least k and at most max(k, enough) of kk[0, n) (shared memory,
+// k <= n) do not exceed, ties of the k-th apart: radix selection from the
+// highest byte in which the keys differ, which ends as soon as the keys up to
+// the k-th's bucket are no more than enough (usually after one pass or two, of
+// up to eight).  Every thread of the CTA calls it with the smallest and
+// largest of the keys it wrote.
+__device__ unsigned long long radix_kth(const unsigned long long *kk, int64_t n, int32_t k, int32_t enough,
+                                        uint64_t mn, uint64_t mx)
 {
     __shared__ unsigned int hist[256];
     __shared__ unsigned long long prefix;
-    __shared__ long long rank;
+    __shared__ long long rank, after;
     __shared__ unsigned long long wmin[32], wmax[32];
     __shared__ int shift0;
     if (threadIdx.x == 0) rank = k - 1;
@@ -196,8 +216,9 @@ __device__ unsigned long long radix_kth(const unsigned long long *kk, int64_t n,
             if ((v & hi) == pre) atomicAdd(&hist[(v >> shift) & 255u], 1u);
         }
         __syncthreads();
-        if (threadIdx.x < 32) pick_digit(hist, shift, prefix, rank);
+        if (threadIdx.x < 32) pick_digit(hist, shift, prefix, rank, after);
         __syncthreads();
+        if (k - 1 + after <= enough) return prefix | ((1ull << shift) - 1);
     }
     return prefix;
 }
@@ -224,7 +245,7 @@ kth_kernel(wf_eval_out res, int64_t P, int32_t k, void *scr)
         mn = min(mn, x);
         mx = max(mx, x);
     }
-    const unsigned long long T = radix_kth(v, n, k, mn, mx);
+    const unsigned long long T = radix_kth(v, n, k, min(2 * k, n), mn, mx);
     if (threadIdx.x == 0) atomicMin(s.T, T);
 }
 
@@ -246,16 +267,19 @@ __device__ void bitonic_sort(Cand *t, int len)
     __syncthreads();
 }
 
+__device__ __forceinline__ void write_one(const Cand &c, int u, int32_t *ids, int64_t *keys, int64_t sa)
+{
+    ids[u] = c.id;
+    if (keys) {
+        keys[3 * u] = c.mk;
+        keys[3 * u + 1] = sa * c.p95;
+        keys[3 * u + 2] = c.gpu;
+    }
+}
+
 __device__ void write_first(const Cand *t, int32_t k, int32_t *ids, int64_t *keys, int64_t sa)
 {
-    for (int u = threadIdx.x; u < k; u += blockDim.x) {
-        ids[u] = t[u].id;
-        if (keys) {
-            keys[3 * u] = t[u].mk;
-            keys[3 * u + 1] = sa * t[u].p95;
-            keys[3 * u + 2] = t[u].gpu;
-        }
-    }
+    for (int u = threadIdx.x; u < k; u += blockDim.x) write_one(t[u], u, ids, keys, sa);
 }
 
 // Items to rank: the plans of an evaluated batch, or the candidates
@@ -298,8 +322,8 @@ __device__ void fold_sort(const Src &src, int64_t n, int32_t k, const unsigned l
 }
 
 // The k best of src[0, n) (k <= n <= kOneCta): the 64-bit keys staged in kk,
-// T the exact k-th smallest of them, the items with keys at most T gathered
-// into t and sorted there by the full key.
+// T a bound that about k of them do not exceed, the items with keys at most T
+// gathered into t and ranked there by the full key.
 template <class Src>
 __device__ void select_and_sort(const Src &src, int64_t n, int32_t k, unsigned long long *kk, Cand *t,
                                 int32_t *ids, int64_t *keys, int64_t sa)
@@ -313,7 +337,7 @@ __device__ void select_and_sort(const Src &src, int64_t n, int32_t k, unsigned l
         mn = min(mn, v);
         mx = max(mx, v);
     }
-    const unsigned long long T = radix_kth(kk, n, k, mn, mx);
+    const unsigned long long T = radix_kth(kk, n, k, max(k, kFew), mn, mx);
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
         if (kk[i] > T) continue;
         const unsigned int slot = atomicAdd(&m, 1u);
@@ -323,6 +347,24 @@ __device__ void select_and_sort(const Src &src, int64_t n, int32_t k, unsigned l
     const unsigned int cnt = m;
     if (cnt > (unsigned)kTile) {  // massive ties with T
         fold_sort(src, n, k, kk, T, t, ids, keys, sa);
+        return;
+    }
+    if (cnt <= (unsigned)kFew) {
+        // Few candidates: a lane's count of those before its own is its place
+        // (the plan index makes every key distinct), with no barrier between
+        // the steps of a sorting network.
+        const int parts = (int)(blockDim.x / kFew), part = threadIdx.x / kFew, i = threadIdx.x % kFew;
+        __shared__ int place[kFew];
+        if (threadIdx.x < kFew) place[threadIdx.x] = 0;
+        __syncthreads();
+        if (i < (int)cnt) {
+            const Cand c = t[i];
+            int ahead = 0;
+            for (int j = part; j < (int)cnt; j += parts) ahead += before(t[j], c);
+            atomicAdd(&place[i], ahead);
+        }
+        __syncthreads();
+        if (part == 0 && i < (int)cnt && place[i] < k) write_one(t[i], place[i], ids, keys, sa);
         return;
     }
     int len = 64;

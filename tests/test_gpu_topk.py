@@ -113,3 +113,19 @@ def test_paths_alternate_on_one_context():
         want_ids, want_keys = oracle.topk(mk[:n], zeros[:n], zeros[:n], st[:n], k)
         assert np.array_equal(ids.cpu().numpy(), want_ids) and np.array_equal(keys.cpu().numpy(), want_keys)
     ctx.close()
+
+
+@pytest.mark.parametrize("P,k", [(1, 1), (128, 128), (129, 127), (129, 129), (300, 128), (1024, 8), (4097, 100), (16384, 200), (20000, 128),
+                                 (20000, 130)])
+@pytest.mark.parametrize("spread", [1, 3, 1 << 20, 1 << 50])
+def test_candidates_around_the_ranking_limit(P, k, spread):
+    """Batches whose selection ends with about 128 candidates (ranked by
+    comparison, or sorted beyond), with few and with many different keys."""
+    rng = np.random.default_rng(P + k)
+    cols = [rng.integers(0, spread, P), rng.integers(0, 4, P), rng.integers(0, 4, P)]
+    status = (rng.random(P) < 0.1).astype(np.uint32)
+    for c in cols:
+        c[status != 0] = np.iinfo(np.int64).max
+    ids, keys = run_topk(*cols, status, k)
+    wids, wkeys = oracle.topk(*cols, status, k)
+    assert np.array_equal(ids, wids) and np.array_equal(keys, wkeys)
