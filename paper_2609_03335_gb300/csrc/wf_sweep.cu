@@ -1013,9 +1013,10 @@ nextuse_kernel(wf_dev_problem dp, wf_plans pl, const uint32_t *status, uint16_t 
 
 // Status bits of every plan (Eq. 8-10), one warp per plan.  Four nodes per
 // lane check placement and fit (one fit mask per node); the warp scatters the
-// inverse of the dispatch sequence (u16 positions) into shared memory and
-// reads it back: a repeated node leaves some position with another position's
-// entry, so every in-range sequence that reads back intact is a permutation.
+// inverse of the dispatch sequence (u16 positions) into empty cells of shared
+// memory: a repeated node leaves a cell empty, so every in-range sequence
+// that fills them all is a permutation.  (Reading the sequence again and
+// comparing every entry: 60.5 us at 16,384 plans of N = 2,000; so 50.8.)
 // The edges (pred | succ << 16) are then checked 32 at a time.  Invalid plans
 // get INT64_MAX metrics here; the sweep skips them.
 __host__ __device__ inline uint32_t status_warp_bytes(int32_t N)
@@ -1048,8 +1049,11 @@ status_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out)
         // Every loop issues kU 16-byte reads per lane before it uses any: on
         // long rows a warp keeps a plan's reads in flight rather than one
         // round trip per 512 bytes (kU = 1 on short rows, whose loops run once).
-        // The inverse permutation, 8 dispatch entries a lane at a time, then
-        // read back: a repeated node leaves some entry unmatched.
+        // The inverse permutation, 8 dispatch entries a lane at a time, into
+        // cells that held no position before: N entries leave a cell empty
+        // exactly when one repeats another (or is out of range).
+        for (int32_t b8 = 8 * lane; b8 < N; b8 += 256) *(uint4 *)(pos + b8) = make_uint4(~0u, ~0u, ~0u, ~0u);
+        __syncwarp();
         for (int32_t b8 = 8 * lane; b8 < N; b8 += kU * 256) {
             uint4 ow[kU];
 #pragma unroll
@@ -1070,20 +1074,13 @@ status_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out)
             }
         }
         __syncwarp();
-        for (int32_t b8 = 8 * lane; b8 < N; b8 += kU * 256) {
-            uint4 ow[kU];
+        for (int32_t b8 = 8 * lane; b8 < N; b8 += 256) {
+            const uint4 c = *(const uint4 *)(pos + b8);
+            const uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-            for (int u = 0; u < kU; ++u)
-                ow[u] = b8 + 256 * u < N ? __ldg((const uint4 *)(order + b8 + 256 * u)) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int32_t i8 = b8 + 256 * u;
-                const uint32_t w[4] = {ow[u].x, ow[u].y, ow[u].z, ow[u].w};
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t h = (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-                    if (i8 + j < N && h < (uint32_t)N && pos[h] != (uint16_t)(i8 + j)) st |= WF_ST_PERMUTATION;
-                }
+            for (int j = 0; j < 4; ++j) {  // (cells at and beyond N stay empty; a position is below 0xFFFF)
+                const bool lo = (w[j] & 0xFFFFu) == 0xFFFFu && b8 + 2 * j < N, hi = (w[j] >> 16) == 0xFFFFu && b8 + 2 * j + 1 < N;
+                if (lo || hi) st |= WF_ST_PERMUTATION;
             }
         }
         st = __reduce_or_sync(0xFFFFFFFFu, st);
