@@ -78,15 +78,15 @@ def topk_launches(P: int, k: int) -> int:
 
 
 def kernel_code(files: dict) -> str:
-    """The evaluation kernels' code from the sources {name: text}: wf_eval.cu
-    and wf_sweep.cu whole, and of wf_internal.cuh the device problem record
+    """The evaluation kernels' code from the sources {name: text}: wf_eval.cu,
+    wf_sweep.cu, wf_stoch.cu and wf_play.cuh whole, and of wf_internal.cuh the device problem record
     and the #defines (the rest of that header is host-side: the context
     record and the launchers' declarations); comments, indentation and blank
     lines removed.  (No string literal in these files holds a comment marker.)"""
     import re
     hdr = files["wf_internal.cuh"]
     rec = re.search(r"struct wf_dev_problem \{.*?\n\};", hdr, flags=re.S)
-    parts = [files["wf_eval.cu"], files["wf_sweep.cu"], rec.group(0) if rec else hdr,
+    parts = [files["wf_eval.cu"], files["wf_sweep.cu"], files["wf_stoch.cu"], files["wf_play.cuh"], rec.group(0) if rec else hdr,
              "\n".join(ln for ln in hdr.splitlines() if ln.startswith("#define"))]
     out = []
     for src in parts:
@@ -100,7 +100,7 @@ def kernel_source_hash() -> str:
     to host-side declarations keeps the recorded counters, any edit to the
     kernels' code drops them."""
     files = {}
-    for f in ("wf_eval.cu", "wf_sweep.cu", "wf_internal.cuh"):
+    for f in ("wf_eval.cu", "wf_sweep.cu", "wf_stoch.cu", "wf_play.cuh", "wf_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2609_03335_gb300", "csrc", f), encoding="utf-8") as fh:
             files[f] = fh.read()
     return hashlib.sha256(kernel_code(files).encode()).hexdigest()[:16]
@@ -709,7 +709,7 @@ def run_gpu(args, rank, world, local):
                          "frac": achieved / peak if peak else None,
                          "traffic": traffic,
                          "kernel": ("wf_eval_plans = status_kernel + pc_kernel (u32 times) + pc_kernel (u64 "
-                                    "times, hand-offs) + eval_list_kernel") if prob.S == 0 else
+                                    "times, hand-offs) + eval_warp_kernel") if prob.S == 0 else
                                    "wf_eval_plans = status_kernel + stoch_kernel + eval_stoch_kernel (hand-offs)",
                          "algorithmic_bytes_per_plan": bpp, "kernel_ms": eval_ms_mean,
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy)" if peak else None},

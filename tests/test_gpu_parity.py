@@ -158,7 +158,7 @@ def test_random_stochastic_windows(seed):
 @pytest.mark.parametrize("S", [1, 2, 31, 63, 64, 65])
 def test_stochastic_sample_counts(S):
     """Sample counts around the width of the per-plan sample block (64 lanes)
-    and beyond it (the int64 path evaluates S > 64)."""
+    and beyond it."""
     rng = np.random.default_rng(4200 + S)
     prob = random_problem(rng, n_sessions=4, D=3)
     r, c, e = wfgen.box_muller_tables()
