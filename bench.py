@@ -564,7 +564,7 @@ def static_timing(wf, prob, plans, dev, flush, reps=5):
     ms = float(np.median(ts))
     return {"plans": fit, "ms": ms, "plans_per_s": fit / (ms * 1e-3),
             "timing": f"median of {reps} calls, L2 flushed before each",
-            "note": "the largest batch of this window the 32 MiB static scratch holds; a thread per plan"}
+            "note": "the largest batch of this window the 32 MiB static scratch holds; a warp per plan"}
 
 
 def run_gpu(args, rank, world, local):
