@@ -275,9 +275,11 @@ int wf_ctx_reserve_host(wf_ctx *ctx);
  * times, loads and arrivals, weights and capacities >= 1 and peak >= weight;
  * when it fails, every plan of the batch gets status WF_ST_TABLES and
  * INT64_MAX metrics, and wf_static_status reports it.  (Acyclicity,
- * duplicate or cross-session edges and "every activation fits somewhere" are
- * not checked: the caller guarantees them, as wf_problem_check does for a
- * context; pred_off[N] must be the length of pred_idx.)
+ * duplicate or cross-session edges, sessions without an activation and
+ * "every activation fits somewhere" are not checked: the caller guarantees
+ * them, as wf_problem_check does for a context; pred_off[N] must be the length
+ * of pred_idx.  A session without an activation counts with a latency of
+ * INT64_MIN - arrival, wrapping.)
  * Scratch is a 32 MiB file-scope device array that every GPU loading this
  * library holds until the process exits.  A call needs 256 B, plus three
  * tables of 4*N bytes each rounded up to 256 B, plus one state row per plan

@@ -145,8 +145,10 @@ __device__ __forceinline__ uint2 settle_lru(Q &q, uint32_t &n, uint32_t &u_d, ui
 
 // The r-th smallest (0-based) of n values a.get(i), by a whole warp.  The p95's rank is near the top (the
 // (n - r)-th largest: 4th of 64, 13th of 256), so the warp takes maxima: the
-// largest value below the last maximum and how many equal it, until the
-// count reaches n - r.  For a rank further down, a radix selection from the
+// largest value up to a bound, first ~0 and then one below the last maximum,
+// and how many equal it, until the count reaches n - r.  (Every step counts at
+// least one value, whatever the values are: when the maximum is 0, all that
+// are left are 0, and enough of them.)  For a rank further down, a radix selection from the
 // highest bit set in any value, each bit decided by a ballot.  Up to 32
 // kCache values are read once into registers (a column of the slot array is
 // a strided read with bank conflicts); more are read again for every step.
@@ -180,12 +182,12 @@ __device__ uint64_t warp_select(const SA &a, int32_t n, int32_t r)
         c[j] = cached && i < n ? (uint64_t)a.get(i) : 0ull;
     }
     if (n - r <= kMaxSteps) {
-        int32_t need = n - r;  // the need-th largest of the values below thr
-        uint64_t thr = ~0ull;
+        int32_t need = n - r;  // the need-th largest of the values up to top
+        uint64_t top = ~0ull;
         for (;;) {
             uint64_t mx = 0;
             each_value(a, n, cached, c, [&](uint64_t v, bool) {
-                if (v < thr) mx = max(mx, v);
+                if (v <= top) mx = max(mx, v);
             });
             const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(mx >> 32));
             const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(mx >> 32) == hi ? (uint32_t)mx : 0u);
@@ -196,7 +198,7 @@ __device__ uint64_t warp_select(const SA &a, int32_t n, int32_t r)
             });
             if (cnt >= need) return m;
             need -= cnt;
-            thr = m;
+            top = m - 1;
         }
     }
     uint64_t any = 0;

@@ -162,3 +162,31 @@ def test_static_entry_on_edges(sessions, sizes, D, M, scale):
         assert want[0][want[3] == 0].max() > 1 << 32
     for a, b in zip(out.numpy(), want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("others", [[1] * 19, [1] * 3 + [0] * 16, [0] * 19, [3, 2, 1, 1, 0, 0], [1] * 250 + [2] * 60 + [0] * 5,
+                                    [1] * 900 + [0] * 200])
+def test_static_entry_with_sessions_that_own_no_activation(others):
+    """Sessions that no activation belongs to, which the device check does not
+    look for: their latency is INT64_MIN - arrival in wrapping 64-bit
+    arithmetic (so INT64_MAX for an arrival of 1, the largest value there is),
+    and the p95 is still the nearest rank of all sessions' values -- ranks near
+    the top and, with many sessions, further down."""
+    from randprob import random_problem
+    from paper_2609_03335_gb300 import build, wf
+    build.build()
+    one = random_problem(np.random.default_rng(8), n_sessions=1, sizes=(6, 6), D=2, M=3).with_(arrival_us=np.zeros(1, np.int64))
+    prob = one.with_(W=1 + len(others), arrival_us=np.r_[0, others].astype(np.int64))
+    plans = wfgen.make_plans(one, 70, 4)
+    mk, lat, gpu, st = oracle.eval_plans(one, plans)
+    out = wf.Results(plans.P)
+    wf.wf_eval_plans_static(wf.DeviceProblem(prob), wf.DevicePlans.from_host(plans, "cuda"), out)
+    wf.wf_static_status()
+    lo = np.full(len(others), np.iinfo(np.int64).min)
+    with np.errstate(over="ignore"):
+        none = lo - np.array(others, np.int64)
+    assert (st == 0).all() and (1 not in others or none.max() == wf.INT64_MAX)
+    rank = (95 * prob.W + 99) // 100 - 1
+    want = np.sort(np.c_[np.tile(none, (plans.P, 1)), lat], axis=1)[:, rank]
+    for a, b in zip(out.numpy(), (mk, want, gpu, st)):
+        assert np.array_equal(a, b)
