@@ -159,7 +159,9 @@ construct_kernel(wf_dev_problem dp, wf_plans out, uint64_t seed, int64_t jitter,
         while (__any_sync(kAll, nready > 0)) {
             const bool act = nready > 0;
             // RankReady: the smallest key (keys are unique).  Its lane then
-            // holds its place, which takes the last entry.
+            // holds its place, which takes the last entry.  (When it was the
+            // last entry nothing moves: the successors' keys go there below,
+            // from other lanes.)
             uint64_t best = ~0ull;
             int32_t at = 0;
             for (int32_t i = g; i < nready; i += 4 * kL) {
@@ -175,7 +177,7 @@ construct_kernel(wf_dev_problem dp, wf_plans out, uint64_t seed, int64_t jitter,
             if (act) --nready;
             const uint64_t tail_key = act ? s.key[nready] : 0ull;
             __syncwarp();
-            if (act && mine == best) s.key[at] = tail_key;
+            if (act && mine == best && at != nready) s.key[at] = tail_key;
             const int32_t u = act ? (int32_t)(best & 0xFFFFu) : 0;
             const uint64_t hu = mix64(hp ^ (uint64_t)u);
             const int64_t rel = (int64_t)((best >> 16) - rank_jitter(hu));
@@ -255,6 +257,7 @@ construct_kernel(wf_dev_problem dp, wf_plans out, uint64_t seed, int64_t jitter,
             // of the session waits for).
             int32_t e = 0, e1 = 0;
             if (on) { e = __ldg(dp.succ_off + tail) + g; e1 = __ldg(dp.succ_off + tail + 1); }
+            __syncwarp();  // (orders the move above before the appended keys)
             do {
                 bool take = false;
                 uint64_t key = 0;

@@ -77,3 +77,15 @@ def test_lanes_per_plan(D, M, P):
     got, res = build(prob, P, seed=3, jitter=5000, plan_base=11)
     want, ends = oracle.construct(prob, P, seed=3, jitter=5000, plan_base=11)
     check(prob, got, res, want, ends)
+
+
+@pytest.mark.parametrize("lengths,D,P", [([1], 1, 3), ([40], 3, 20000), ([25, 2], 12, 9000), ([12, 1, 1], 20, 5000)])
+def test_the_last_ready_entry_is_taken(lengths, D, P):
+    """Chains: the ready set holds one node or a few, so the node taken is often
+    its last entry, whose place the next ready node takes at once -- over enough
+    plans that every lane group builds a second one in the same scratch."""
+    from test_gpu_edges import chains_window
+    prob = chains_window(lengths, D=D, M=2, seed=len(lengths))
+    got, res = build(prob, P, seed=2, jitter=300, plan_base=1)
+    want, ends = oracle.construct(prob, P, seed=2, jitter=300, plan_base=1)
+    check(prob, got, res, want, ends)
