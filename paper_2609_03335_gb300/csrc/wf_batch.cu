@@ -381,6 +381,7 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
             out.gpu_us[p] = g_all + (int64_t)n_open * (int64_t)end;
         }
     }
+    __syncwarp();  // every lane reads the latencies that a plan's lanes wrote
     // The p95 (Section 4.2, nearest rank) of the warp's plans, one after the other.
     const int32_t rank = (int32_t)((95 * (int64_t)W + 99) / 100 - 1);
     for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, done && g == 0); todo; todo &= todo - 1) {

@@ -79,6 +79,18 @@ def test_lanes_per_plan(D, M, B, P):
     assert_same(_gpu(prob, plans), oracle_eval(prob, plans))
 
 
+@pytest.mark.parametrize("sessions,D,B", [(1, 3, 2), (33, 8, 4), (100, 12, 4), (300, 5, 3), (700, 20, 1)])
+def test_p95_over_every_lane_s_sessions(sessions, D, B):
+    """A plan's lanes write its sessions' latencies side by side and the whole
+    warp then selects among them: fewer sessions than lanes, several a lane,
+    more than the selection keeps in registers (256), and a rank beyond its
+    taking of maxima (700: the 36th largest)."""
+    rng = np.random.default_rng(sessions)
+    prob = random_problem(rng, n_sessions=sessions, sizes=(4, 5), D=D, M=4).with_(batch=B)
+    plans = wfgen.make_plans(prob, 61, 2)
+    assert_same(_gpu(prob, plans), oracle_eval(prob, plans))
+
+
 @pytest.mark.parametrize("scale,B", [(165000, 2), (1 << 20, 4), (1 << 20, 6), (1 << 24, 1)])
 def test_times_past_32_bits(scale, B):
     """Some or all plans leave the 32-bit sweep (and with the largest scale
