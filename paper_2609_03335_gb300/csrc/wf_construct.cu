@@ -77,9 +77,17 @@ __host__ __device__ inline size_t scratch_bytes(int32_t N)
 }
 
 // Minimum of a 64-bit key over the kL lanes of a group.
+// A whole warp: the high halves, then the low halves of those that hold it
+// (five shuffles of 64 bits instead: 16,384 plans of N = 1,000, D = 32 in
+// 9.07 ms, so 7.94).
 template <int kL>
 __device__ __forceinline__ uint64_t group_min(uint64_t key)
 {
+    if constexpr (kL == 32) {
+        const uint32_t hi = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)(key >> 32));
+        const uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, (uint32_t)(key >> 32) == hi ? (uint32_t)key : 0xFFFFFFFFu);
+        return ((uint64_t)hi << 32) | lo;
+    }
 #pragma unroll
     for (int o = kL / 2; o; o >>= 1) {
         const uint64_t other = __shfl_xor_sync(0xFFFFFFFFu, key, o);
