@@ -18,10 +18,12 @@
 // reclamation, Eq. 11; loads, Eq. 5; starts and finishes, Eq. 2, 7, 10), so
 // the constructor's timeline is the one wf_eval_plans reports for its plan.
 //
-// A plan is built by a group of 8, 16 or 32 lanes (the device count), so a
-// warp builds 4, 2 or 1 plans side by side: a plan's steps are a serial chain
-// of small parallel parts -- the ready set's minimum, a score per device, a
-// few successors -- which fill 8 lanes and leave most of 32 idle.  Lane g
+// A plan is built by a group of 8, 16 or 32 lanes (at least the device
+// count), so a warp builds 4, 2 or 1 plans side by side: a plan's steps are a
+// serial chain of small parallel parts -- the ready set's minimum, a score per
+// device, a few successors -- which fill 8 lanes and leave most of 32 idle.  A
+// batch that leaves the chip's warps idle takes more lanes instead, which
+// shorten the chain (lanes_of).  Lane g
 // keeps device g's state in registers (free time, residency queue, resident
 // weights).  Control flow is uniform over the warp: a loop runs until every
 // plan of the warp is through.  Bound by integer issue (64-bit hashes, keys
@@ -38,7 +40,18 @@ constexpr int kWarps = 4;          // warps per CTA
 constexpr int kCtasPerSm = 7;      // resident CTAs per SM (72 registers per thread)
 constexpr int kWarpsPerSm = kWarps * kCtasPerSm;
 
-int lanes_of(int32_t D) { return D <= 8 ? 8 : D <= 16 ? 16 : 32; }  // lanes per plan
+// Lanes per plan.  The chain of one plan is shorter on more lanes (a warp's
+// minimum is two reductions, a longer ready set takes fewer rounds), the
+// chip's issue slots hold more plans on fewer.  N = 1,000, D = 3, us with 8,
+// 16, 32 lanes: 512 plans 1,267, 1,128, 928; 1,024: 1,278, 1,130, 988; 2,048: 1,291,
+// 1,234, 1,311; 3,072: 1,535, 1,450, 1,804; 4,096: 1,588, 1,676, 2,075.  N = 40 to
+// 2,000 with 3 and 8 devices change sides at the same batches, 8 and 24 plans an
+// SM.
+int lanes_of(int32_t D, int64_t P, int sms)
+{
+    const int least = D <= 8 ? 8 : D <= 16 ? 16 : 32;
+    return std::max(least, P <= 8 * (int64_t)sms ? 32 : P <= 24 * (int64_t)sms ? 16 : 8);
+}
 
 __device__ __forceinline__ uint64_t mix64(uint64_t x)  // SplitMix64 output function
 {
@@ -290,21 +303,20 @@ construct_kernel(wf_dev_problem dp, wf_plans out, uint64_t seed, int64_t jitter,
     }
 }
 
-// Plans built at once: as many as are resident, as far as 1 GiB of scratch
-// goes (112 plans per SM up to N of about 3,500), and at least 60 per SM
-// beyond that.
+// Plans built at once by the largest batch: as many as are resident, as far as
+// 1 GiB of scratch goes (112 plans per SM up to N of about 3,500), and at least
+// 60 per SM beyond that (more than a batch on more lanes holds at all).
 int64_t plans_at_once(const wf_ctx *c)
 {
     const int64_t fit = ((int64_t)1 << 30) / (int64_t)scratch_bytes(c->dp.N);
-    const int64_t resident = (int64_t)kWarpsPerSm * (32 / lanes_of(c->dp.D));
+    const int64_t resident = (int64_t)kWarpsPerSm * (32 / lanes_of(c->dp.D, c->max_P, c->sms));
     return std::min<int64_t>(c->max_P, std::min<int64_t>(c->sms * resident, std::max<int64_t>(fit, (int64_t)c->sms * 60)));
 }
 
-// Calls f(kernel) for this problem's instantiation.
+// Calls f(kernel) for this problem's instantiation with l lanes per plan.
 template <typename F>
-int construct_visit(const wf_dev_problem &dp, F &&f)
+int construct_visit(const wf_dev_problem &dp, int l, F &&f)
 {
-    const int l = lanes_of(dp.D);
     if (dp.M <= 8)
         return l == 8 ? f(construct_kernel<uint32_t, 8>) : l == 16 ? f(construct_kernel<uint32_t, 16>)
                                                                    : f(construct_kernel<uint32_t, 32>);
@@ -334,11 +346,12 @@ extern "C" int wf_construct_plans(wf_ctx *c, const wf_plans *out, uint64_t seed,
         if (rc) { c->construct_scratch = nullptr; return rc; }
     }
     const int64_t slots = std::min<int64_t>(out->P, c->construct_threads);
-    const int64_t per_cta = kWarps * (32 / lanes_of(dp.D));
+    const int lanes = lanes_of(dp.D, out->P, c->sms);
+    const int64_t per_cta = kWarps * (32 / lanes);
     const unsigned blocks = (unsigned)((slots + per_cta - 1) / per_cta);
     const uint64_t jd = (uint64_t)jitter_us + 1;
     const Mod64 jm = {~0ull / jd, jd};
-    return construct_visit(dp, [&](auto k) {
+    return construct_visit(dp, lanes, [&](auto k) {
         k<<<blocks, 32 * kWarps, 0, (cudaStream_t)stream>>>(dp, *out, seed, jitter_us, jm,
                                                             (uint8_t *)c->construct_scratch, slots);
         return wf_cuda_check(cudaGetLastError(), "construct launch");

@@ -89,3 +89,26 @@ def test_the_last_ready_entry_is_taken(lengths, D, P):
     got, res = build(prob, P, seed=2, jitter=300, plan_base=1)
     want, ends = oracle.construct(prob, P, seed=2, jitter=300, plan_base=1)
     check(prob, got, res, want, ends)
+
+
+@pytest.mark.parametrize("D,M", [(5, 8), (8, 9), (13, 4), (16, 9)])
+def test_lanes_by_batch(D, M):
+    """The batches at which a plan takes 32, 16 or 8 lanes (8 and 24 plans an
+    SM), and one more plan each, on one context made for the largest; the same
+    seed gives the same plans whatever the lanes."""
+    import torch
+    wf = lib()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(D)
+    prob = random_problem(rng, n_sessions=3, sizes=(4, 6), D=D, M=M)
+    most = 24 * sms + 1
+    ctx = wf.Ctx(prob, max_P=most)
+    want, _ = oracle.construct(prob, most, seed=6, jitter=700)
+    for P in (most, 24 * sms, 8 * sms + 1, 8 * sms, 3):
+        out = wf.DevicePlans.empty(P, prob.N)
+        wf.wf_construct_plans(ctx, out, 6, 700)
+        torch.cuda.synchronize()
+        wf.wf_ctx_status(ctx)
+        for g, w in zip(out.numpy(prob.N)[:4], (want.place, want.order, want.fuse, want.prefetch)):
+            assert np.array_equal(g, w[:P]), P
+    ctx.close()
