@@ -249,14 +249,17 @@ kth_kernel(wf_eval_out res, int64_t P, int32_t k, void *scr)
     if (threadIdx.x == 0) atomicMin(s.T, T);
 }
 
-// Sorts t[0, len) ascending; len is a power of two, at most kTile.
+// Sorts t[0, len) ascending; len is a power of two, at most kTile.  The pair's
+// index without a division (stride is a power of two): a search round whose
+// candidates tie by the thousand, 4,096 children of N = 32, 395 us with the
+// division, 364 without.
 __device__ void bitonic_sort(Cand *t, int len)
 {
     for (int size = 2; size <= len; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
             __syncthreads();
             for (int u = threadIdx.x; u < len / 2; u += blockDim.x) {
-                const int i = 2 * stride * (u / stride) + (u % stride);
+                const int i = 2 * u - (u & (stride - 1));  // 2 stride (u / stride) + u % stride
                 const int j = i + stride;
                 const bool up = (i & size) == 0;
                 const Cand a = t[i], b = t[j];
