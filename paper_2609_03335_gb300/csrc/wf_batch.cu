@@ -4,9 +4,9 @@
 // under the limit an admission waits for running units to end, so residency
 // cannot be settled ahead of the times.
 //
-// A play warp holds 32 / kL plans, kL lanes each (8, 16 or 32 by the device
-// count); lane g of a plan is its device g and keeps that device's state in
-// registers: the current replica's model, the last admission, the residency
+// A play warp holds 32 / kL plans, kL lanes each (8 or 16 by the device
+// count); lane g of a plan is its device g, and beyond 16 devices its device g
+// + 16 as well, and keeps that device's state in registers: the current replica's model, the last admission, the residency
 // queue, resident weights and count, the occupancy balance and, up to four of
 // them, the running slots (beyond, those are in shared memory, in the lane's
 // own column).  Every lane walks the chunk's positions; a unit is played by
@@ -39,12 +39,17 @@ constexpr int kBqFull = 1, kBqEmpty = kBqFull + kBqBuffers;  // named barriers
 constexpr int kBqRegs = 4;    // running slots kept in registers
 static_assert(kBqEmpty + kBqBuffers <= 16, "named barriers");
 
-template <int kL>
+template <int kL, int kDev, int kB>
 struct BqShape {
     static constexpr int kPlay = kBqPlans * kL / 32;  // play warps
     static constexpr int kWarps = kPlay + kBqProducers;
-    // Six CTAs of 8-device plans share an SM at 2,000 activations.
-    static constexpr int kMinBlocks = kL == 8 ? 6 : kL == 16 ? 4 : 2;
+    // Six CTAs of 8-device plans share an SM at 2,000 activations.  With two
+    // devices a lane three CTAs do where both devices' running slots are
+    // registers (92 to 96 a thread), else four.  65,536 plans of N = 32, D = 32, B_q =
+    // 1, 4, 8, us: 32 lanes a plan, a device each, 575, 577, 768; 16 lanes, two
+    // devices each, 437, 442, 503 (a lane a plan with its state in shared
+    // memory 487, 537, 751).
+    static constexpr int kMinBlocks = kL == 8 ? 6 : kDev == 1 ? 4 : kB ? 3 : 4;
 };
 
 struct BqLayout {
@@ -72,6 +77,14 @@ __host__ __device__ inline BqLayout bq_layout(int32_t D, int32_t M, int32_t W, i
     l.open = o; o += round16(4u * P);
     l.total = o;
     return l;
+}
+
+template <typename T>
+__device__ __forceinline__ void exchange_if(bool c, T &a, T &b)
+{
+    const T t = a;
+    a = c ? b : a;
+    b = c ? t : b;
 }
 
 // The running slots of one device: each one's end and KV (0 and 0 when free).
@@ -103,6 +116,11 @@ struct Running {  // in registers, B <= kB of them
         for (int j = 0; j < kB; ++j)
             if (j == slot) { e[j] = t; kv[j] = k; }
     }
+    __device__ __forceinline__ void swap_if(bool c, Running &o)
+    {
+#pragma unroll
+        for (int j = 0; j < kB; ++j) { exchange_if(c, e[j], o.e[j]); exchange_if(c, kv[j], o.kv[j]); }
+    }
 };
 template <typename TT>
 struct Running<TT, 0> {  // in the lane's column of shared memory
@@ -128,18 +146,28 @@ struct Running<TT, 0> {  // in the lane's column of shared memory
         e[slot * cols] = t;
         kv[slot * cols] = k;
     }
+    __device__ __forceinline__ void swap_if(bool c, Running &o) { exchange_if(c, e, o.e); exchange_if(c, kv, o.kv); }
+};
+
+// The device of a lane that is not being played, when it has two.
+template <typename Q, typename TT, int kB>
+struct OtherDevice {
+    Q queue = 0;
+    uint32_t n = 0, used = 0, cur = 0xFFFFFFFFu, cap = 0;
+    TT ladm = 0;
+    Running<TT, kB> slots;
 };
 
 // Groups of kBqPlans plans: every plan of the batch (in_list null, a CTA per
 // group) or the listed ones (CTAs walk over groups).
-template <typename Q, int kL, typename TT, typename ST, int kB>
-__global__ void __launch_bounds__(32 * BqShape<kL>::kWarps, BqShape<kL>::kMinBlocks)
+template <typename Q, int kL, int kDev, typename TT, typename ST, int kB>
+__global__ void __launch_bounds__(32 * BqShape<kL, kDev, kB>::kWarps, BqShape<kL, kDev, kB>::kMinBlocks)
 bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_list, const int32_t *in_count,
           int32_t *ovf_list, int32_t *ovf_count)
 {
     constexpr int kP = kBqPlans, kPitch = kBqPitch;
-    constexpr int kPlay = BqShape<kL>::kPlay;
-    constexpr int kThreads = 32 * BqShape<kL>::kWarps;
+    constexpr int kPlay = BqShape<kL, kDev, kB>::kPlay;
+    constexpr int kThreads = 32 * BqShape<kL, kDev, kB>::kWarps;
     constexpr bool kNarrow = sizeof(TT) == 4;
     extern __shared__ __align__(128) uint8_t sm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -238,10 +266,16 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     for (int32_t k = g; k < dp.nslots + 2; k += kL) slots.set(k, 0);
     __syncthreads();
     const uint32_t trash = (uint32_t)dp.nslots;
-    const uint32_t capd = g < D ? (uint32_t)cap[g] : 0u;
+    uint32_t capd = g < D ? (uint32_t)cap[g] : 0u;
     Q queue = 0;                    // resident models, least recently used first
     uint32_t n = 0, used = 0;       // their count and weights
     uint32_t cur = 0xFFFFFFFFu;     // model of the current replica
+    int dev = g;                    // the device whose state this is (of g and g + kL)
+    OtherDevice<Q, TT, kB> other;   // the other one's
+    if constexpr (kDev == 2) {
+        other.slots.init(g + kL < D ? B : 0, (TT *)(sm + L.se) + q * D + g + kL, (uint32_t *)(sm + L.sk) + q * D + g + kL, kP * D);
+        other.cap = g + kL < D ? (uint32_t)cap[g + kL] : 0u;
+    }
     TT ladm = 0, end = 0;           // last admission; latest finish of the lane's units
     int64_t gsum = 0;               // closed occupancy minus the open interval's start
     uint32_t ovf = 0;
@@ -255,7 +289,18 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         for (int32_t k = 0; k < kmax; ++k) {
             const uint2 nw1 = rb[(1 * kChunk + (k + 1 < kmax ? k + 1 : k)) * kPitch];
             const uint32_t r3 = w1.y;
-            if (!(r3 & kSkip) && (int)(r3 & 31u) == g) {
+            if (!(r3 & kSkip) && (int)((r3 & 31u) % (kDev == 1 ? 32 : kL)) == g) {
+                if constexpr (kDev == 2) {  // (by selects: lanes that exchange play together with those that do not)
+                    const bool c = (int)(r3 & 31u) != dev;
+                    exchange_if(c, queue, other.queue);
+                    exchange_if(c, n, other.n);
+                    exchange_if(c, used, other.used);
+                    exchange_if(c, cur, other.cur);
+                    exchange_if(c, capd, other.cap);
+                    exchange_if(c, ladm, other.ladm);
+                    run_slots.swap_if(c, other.slots);
+                    dev = (int)(r3 & 31u);
+                }
                 const uint2 w0 = rb[(0 * kChunk + k) * kPitch], w2 = rb[(2 * kChunk + k) * kPitch];
                 const uint32_t m = (r3 >> 5) & 15u, kv = w1.x;
                 const TT arr = w0.y, run = w0.x;  // run includes the grant
@@ -309,7 +354,7 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 TT start = adm;
                 if (!join) {
                     const TT ls = max(drain, (!hit && (r3 & kPrefetch)) ? arr : rel);
-                    const TT le = ls + (hit ? 0u : (uint32_t)load[m * D + g]);
+                    const TT le = ls + (hit ? 0u : (uint32_t)load[m * D + dev]);
                     if (kNarrow) ovf |= le < ls;
                     start = max(le, rel);
                     adm = ls;
@@ -357,7 +402,7 @@ bq_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     }
     // The plan's results from its lanes.
     int64_t g_all = gsum;
-    uint32_t n_open = n != 0, o_all = ovf;
+    uint32_t n_open = (n != 0) + (kDev == 2 && other.n != 0), o_all = ovf;
     if (kNarrow) o_all |= end == (TT)kRunCap;
 #pragma unroll
     for (int o = kL / 2; o; o >>= 1) {
@@ -415,9 +460,9 @@ int launch_bq(const wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, siz
     const wf_dev_problem &dp = ctx->dp;
     int64_t blocks = (pl->P + kBqPlans - 1) / kBqPlans;
     if (in_list) blocks = std::min<int64_t>(blocks, (int64_t)ctx->sms * 6);
-    auto go = [&](auto q, auto l) {
-        constexpr int kL = decltype(l)::value;
-        const auto k = bq_kernel<typename decltype(q)::type, kL, TT, ST, kB>;
+    auto go = [&](auto q, auto l, auto n) {
+        constexpr int kL = decltype(l)::value, kDev = decltype(n)::value;
+        const auto k = bq_kernel<typename decltype(q)::type, kL, kDev, TT, ST, kB>;
         int rc = wf_cuda_check(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                                "batch sweep smem attribute");
         // The whole of the SM's memory as shared memory: by default four
@@ -425,11 +470,11 @@ int launch_bq(const wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, siz
         if (!rc) rc = wf_cuda_check(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                          cudaSharedmemCarveoutMaxShared), "batch sweep carve-out");
         if (rc) return rc;
-        k<<<(unsigned)blocks, 32 * BqShape<kL>::kWarps, smem, st>>>(dp, *pl, *out, in_list, in_count, list, count);
+        k<<<(unsigned)blocks, 32 * BqShape<kL, kDev, kB>::kWarps, smem, st>>>(dp, *pl, *out, in_list, in_count, list, count);
         return wf_cuda_check(cudaGetLastError(), "batch sweep launch");
     };
-    auto by_q = [&](auto l) { return dp.M <= 8 ? go(Ty<uint32_t>{}, l) : go(Ty<uint64_t>{}, l); };
-    return dp.D <= 8 ? by_q(Iv<8>{}) : dp.D <= 16 ? by_q(Iv<16>{}) : by_q(Iv<32>{});
+    auto by_q = [&](auto l, auto n) { return dp.M <= 8 ? go(Ty<uint32_t>{}, l, n) : go(Ty<uint64_t>{}, l, n); };
+    return dp.D <= 8 ? by_q(Iv<8>{}, Iv<1>{}) : dp.D <= 16 ? by_q(Iv<16>{}, Iv<1>{}) : by_q(Iv<16>{}, Iv<2>{});
 }
 
 int launch_bq64(const wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, size_t smem, const int32_t *in_list,

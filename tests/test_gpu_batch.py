@@ -79,6 +79,18 @@ def test_lanes_per_plan(D, M, B, P):
     assert_same(_gpu(prob, plans), oracle_eval(prob, plans))
 
 
+@pytest.mark.parametrize("D,M,B,P", [(17, 3, 1, 40), (17, 9, 4, 1000), (24, 8, 5, 333), (31, 16, 4, 64), (32, 8, 64, 9), (32, 5, 2, 2000)])
+def test_two_devices_a_lane(D, M, B, P):
+    """Beyond 16 devices a lane plays two of them in turn: windows long enough
+    that both are used and exchanged often, running slots in registers and in
+    shared memory, retain rows, some invalid plans."""
+    rng = np.random.default_rng(D + B)
+    prob = random_problem(rng, n_sessions=60, D=D, M=M).with_(batch=B)
+    plans = wfgen.make_plans(prob, P, 8, p_retain=0.6 if B == 1 else None)
+    inject_invalid(plans, prob, rng)
+    assert_same(_gpu(prob, plans), oracle_eval(prob, plans))
+
+
 @pytest.mark.parametrize("sessions,D,B", [(1, 3, 2), (33, 8, 4), (100, 12, 4), (300, 5, 3), (700, 20, 1)])
 def test_p95_over_every_lane_s_sessions(sessions, D, B):
     """A plan's lanes write its sessions' latencies side by side and the whole
