@@ -1403,14 +1403,14 @@ struct CfgKey {
     }
 };
 
-// The windows that take reclamation by next use: those of which three plans
-// fit a CTA with a lane's state per plan and device (16-bit next uses, a queue
-// word).  The state per model is up to 8 KB larger, so near that limit the
-// 64-bit sweep plays two plans a CTA.
+// The windows that take reclamation by next use, no more and no fewer: those of
+// which three plans fit a CTA with a lane's state per plan and device (16-bit
+// next uses, a queue word).  The state per model is up to 8 KB larger, so near
+// that limit the 64-bit sweep plays two plans a CTA.
 bool next_use_window(const wf_dev_problem &dp)
 {
     const int32_t D = dp.D, M = dp.M;
-    const size_t o = 64 + round16(4u * D) + round16(4u * M * D) + round16(4u * dp.W) + 4608 + round16(24u * (dp.nslots + 2)) +
+    const size_t o = round16(4u * M) + round16(4u * D) + round16(4u * M * D) + round16(4u * dp.W) + 4608 + round16(24u * (dp.nslots + 2)) +
                      round16(24u * D) + round16((M <= 8 ? 12u : 24u) * D) + round16(12u * D) + round16(3u * D) + 32 +
                      round16(6u * D * M) + round16(3u * M) + 48 + (dp.phi_life ? round16(6u * D) : 0u);
     return o <= 227 * 1024;
@@ -1419,7 +1419,7 @@ bool next_use_window(const wf_dev_problem &dp)
 wf_sweep_cfg choose(const wf_dev_problem &dp)
 {
     wf_sweep_cfg c = {};
-    if (!sweep_usable(dp)) return c;
+    if (!sweep_usable(dp) || (dp.reclaim && !next_use_window(dp))) return c;
     const size_t s32 = layout_bytes<kPlans32, uint32_t>(dp);
     c.res32 = resident<uint32_t>(dp, kPlans32, s32);
     if (c.res32 > 0) c.smem32 = s32;
@@ -1440,7 +1440,7 @@ wf_sweep_cfg choose(const wf_dev_problem &dp)
             c.res64 = n;
         }
     }
-    if (!c.smem64 && dp.reclaim && next_use_window(dp)) {
+    if (!c.smem64 && dp.reclaim) {
         const size_t sm = layout_bytes<2, uint64_t>(dp);
         c.res64 = resident<uint64_t>(dp, 2, sm);
         if (c.res64 > 0) {

@@ -97,6 +97,40 @@ def test_tied_and_nearly_tied_quotients(loads, D, M):
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
 
 
+def lone_sessions(W, D, M, seed):
+    """W sessions of one activation each: as many finish slots as sessions."""
+    rng = np.random.default_rng(seed)
+    dev = wfgen.DeviceSpec(cap_gib=[60 + d for d in range(D)], speed=[1.0] * D, bw_gbps=[1] * D)
+    prob = wfgen.assemble("wide", [[("planner", [])] for _ in range(W)], np.sort(rng.integers(0, 500, W)).astype(np.int64), dev,
+                          [5 + m for m in range(M)], rng, lat_median_us=100, lat_sigma=0.6, kv_lo=1, kv_hi=20)
+    prob = prob.with_(model=rng.integers(0, M, W).astype(prob.model.dtype))
+    return prob.with_(peak_mib=np.repeat(prob.weight_mib[prob.model] + 64, D).astype(np.int32))
+
+
+@pytest.mark.parametrize("D,M", [(1, 1), (2, 2), (3, 4), (2, 6), (7, 8), (5, 12), (32, 16)])
+def test_last_window_that_takes_the_policy(D, M):
+    """The windows that take the policy are those whose state for three plans
+    (a queue word and 16-bit next uses per plan and device) fits a CTA's
+    227 KiB, whatever the layout of the sweep that plays them: the largest
+    one takes it and gives the oracle's results, the next refuses it."""
+    wf = lib()
+    r16 = lambda x: (x + 15) & ~15
+    queue = 12 if M <= 8 else 24
+
+    def size(W):
+        return (r16(4 * M) + r16(4 * D) + r16(4 * M * D) + r16(4 * W) + 4608 + r16(24 * (W + 2)) + r16(24 * D) + r16(queue * D) +
+                r16(12 * D) + r16(3 * D) + 32 + r16(6 * D * M) + r16(3 * M) + 48)
+    W = next(w for w in range(9000, 1, -1) if size(w) <= 227 * 1024)
+    prob = lone_sessions(W, D, M, 10 * D + M)
+    plans = wfgen.make_plans(prob, 4, 1)
+    assert_same(gpu_eval(prob.with_(reclaim=1), plans), oracle_eval(prob.with_(reclaim=1), plans))
+    ctx = wf.Ctx(lone_sessions(W + 1, D, M, 10 * D + M), max_P=4)
+    with pytest.raises(wf.WfError) as e:
+        wf.wf_ctx_set_reclaim(ctx, 1)
+    assert e.value.code == wf.WF_EINVAL
+    ctx.close()
+
+
 def test_largest_window():
     """A window near the shared-memory limit of the policy (32 devices, 16
     models, 7,800 sessions), where the sweep plays two plans per CTA."""
