@@ -30,6 +30,7 @@
 // and sums each unit's load delay plus its reload time.
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -65,9 +66,10 @@ struct Ring {
 constexpr int kPairs = 3;
 
 // Lanes per plan of the residency stage under reclamation by next use: kPer
-// models a lane, of the 8 or 16 that a sweep is compiled for.
+// models a lane, of the 4, 8 or 16 that a sweep is compiled for (Q: a word of
+// as many 4-bit model ids).
 template <typename Q>
-constexpr int kPer = sizeof(Q) == 4 ? 1 : 2;
+constexpr int kPer = sizeof(Q) <= 4 ? 1 : 2;
 template <typename Q>
 constexpr int kModelLanes = 2 * (int)sizeof(Q) / kPer<Q>;
 
@@ -280,7 +282,7 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
     l.weight = o; o += 4u * 16;  // (zeros beyond M: read for the queue's empty places)
     l.load = o; o += round16(4u * M * D);
     l.rcost = o; o += kReclaim ? round16(4u * M * D) : 0u;
-    l.wsum = o; o += kReclaim ? 256u * (uint32_t)sizeof(Q) : 0u;  // (256 sums for each eight models)
+    l.wsum = o; o += kReclaim ? 256u * (uint32_t)sizeof(Q) : 0u;  // (the sums of each set of eight models; with Q of 16 bits more than the 16 used)
     l.arr = o; o += round16(4u * W);
     l.ring = o; o += round16(8u * Ring<kReclaim>::kBuffers * kPairs * kChunk * PcShape<kP>::kPitch);
     l.next = o; o += kReclaim ? round16(2u * Ring<kReclaim>::kBuffers * kChunk * PcShape<kP>::kPitch) : 0u;
@@ -290,7 +292,8 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
     const uint32_t rs = (uint32_t)(G::rows(D) * G::kLanes);
     // Residency state: a word per device (DevState), or under reclamation by
     // next use a word per (device, model), and the free capacity apart.
-    l.queue = o; o += round16((kReclaim ? 4u * kPer<Q> : (uint32_t)sizeof(DevState<Q>)) * rs);
+    using State = std::conditional_t<kReclaim != 0, uint32_t[kPer<Q>], DevState<Q>>;
+    l.queue = o; o += round16((uint32_t)sizeof(State) * rs);
     l.free = o; o += kReclaim ? round16(4u * D * kP) : 0u;
     l.open = o; o += round16(4u * kP);
     l.flag = o; o += 16;
@@ -303,6 +306,8 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
 template <int kP, typename TT, int kReclaim = 0, bool kPhi = false, typename ST = TT>
 inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, int32_t NS)
 {
+    if constexpr (kReclaim != 0)
+        if (M <= 4) return pc_layout_q<kP, TT, uint16_t, kReclaim, kPhi, ST>(D, M, W, NS);
     return M <= 8 ? pc_layout_q<kP, TT, uint32_t, kReclaim, kPhi, ST>(D, M, W, NS)
                   : pc_layout_q<kP, TT, uint64_t, kReclaim, kPhi, ST>(D, M, W, NS);
 }
@@ -532,8 +537,8 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         } else {
         // Reclamation by next use counts a model's copies over all devices, so
         // a plan's units are played one after another, by kL lanes that each
-        // stand for two models (l and l + kL): a lane keeps the number of each
-        // one's copies and, in shared memory, per device the copy's next use
+        // stand for a model, or beyond eight models for two (l and l + kL): a
+        // lane keeps the number of each one's copies and, in shared memory, per device the copy's next use
         // and its last use (0: not resident).  Victims go one at a time: a copy
         // also resident elsewhere first, then the largest (next use -
         // position) / reload cost (no next use or a free reload: infinite),
@@ -547,6 +552,10 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         // scanned the queue for each victim, 4,095; a lane per model 2,722; two
         // models a lane (270 instructions for eight plans, half the warps) 3,010;
         // a lane per model with a loop that takes one victim at a time 3,172.
+        // Up to four models half the lanes would idle: four lanes a plan, two
+        // residency warps.  56,387 plans of N = 376, D = 4, M = 2: a lane per plan
+        // 963, eight lanes 1,171, four 897; 5,629 of N = 2,250, D = 2, M = 3: 760,
+        // 912, 734.
         constexpr int kL = kModelLanes<Q>;
         constexpr int kI = kPer<Q>;
         constexpr uint32_t kAll = (1u << kL) - 1u;
@@ -1240,11 +1249,15 @@ int launch_pc(const wf_dev_problem &dp, int sms, int resident, const wf_plans *p
 template <typename TT, int kR, typename F>
 int pc_visit(const wf_dev_problem &dp, int kp, F &&f)
 {
+    auto by_q = [&](auto p, auto s) {
+        if constexpr (kR != 0)
+            if (dp.M <= 4) return f(Ty<uint16_t>{}, p, s);
+        return dp.M <= 8 ? f(Ty<uint32_t>{}, p, s) : f(Ty<uint64_t>{}, p, s);
+    };
     if constexpr (sizeof(TT) == 4) {  // the u32 sweep has one shape
         (void)kp;
-        return dp.M <= 8 ? f(Ty<uint32_t>{}, Iv<kPlans32>{}, Ty<TT>{}) : f(Ty<uint64_t>{}, Iv<kPlans32>{}, Ty<TT>{});
+        return by_q(Iv<kPlans32>{}, Ty<TT>{});
     } else {
-        auto by_q = [&](auto p, auto s) { return dp.M <= 8 ? f(Ty<uint32_t>{}, p, s) : f(Ty<uint64_t>{}, p, s); };
         auto by_p = [&](auto s) {
             if constexpr (kR != 0)
                 if (kp == 2) return by_q(Iv<2>{}, s);

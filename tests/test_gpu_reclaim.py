@@ -97,6 +97,21 @@ def test_tied_and_nearly_tied_quotients(loads, D, M):
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
 
 
+@pytest.mark.parametrize("D,M,P,scale", [(1, 1, 5, 1), (4, 2, 333, 1), (3, 3, 200, 1), (9, 4, 100, 1), (32, 4, 33, 1), (3, 5, 100, 1),
+                                         (2, 4, 100, 150000), (4, 1, 100, 1 << 20)])
+def test_few_models(D, M, P, scale):
+    """Four lanes a plan up to four models (and five models on eight lanes),
+    with retain rows, invalid plans and run times that leave 32 bits."""
+    rng = np.random.default_rng(3400 + 10 * D + M)
+    prob = random_problem(rng, n_sessions=12, sizes=(6, 12), D=D, M=M)
+    prob = prob.with_(reclaim=1, lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, (1 << 28)).astype(np.int32))
+    plans = wfgen.make_plans(prob, P, M, p_retain=0.7 if D % 2 else None)
+    if P > 8:
+        plans.place[3, 1] = D
+        plans.order[5, 0] = plans.order[5, 1]
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
+
+
 def lone_sessions(W, D, M, seed):
     """W sessions of one activation each: as many finish slots as sessions."""
     rng = np.random.default_rng(seed)
