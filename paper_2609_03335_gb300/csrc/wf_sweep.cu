@@ -966,9 +966,17 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
 // the same model (0xFFFF: none).  A warp per plan walks its positions from the
 // end, 32 at a time; lanes with equal (device, model) keys find each other
 // with __match_any_sync, and a shared table carries the first occurrence of
-// each key to the chunk before.
+// each key to the chunk before.  On windows of several chunks (kDeep) three
+// chunks of gathers are in flight ahead of the one being settled; one or two
+// chunks have nothing to run ahead of, and what bounds those is the plans an
+// SM holds: 32 registers instead of 48, no read for a position that is not
+// there.  39,692 plans of N = 22, us: 18.3 with the deep form, 12.0 without; the
+// call on 30,000 plans of N = 32, D = M = 8 137 and 134, of N = 64 212 and 209, and
+// from N = 128 on the deep form is ahead (355 and 359).
 constexpr int kNuWarps = 4;
+constexpr int32_t kNuShort = 64;  // activations
 
+template <bool kDeep>
 __global__ void __launch_bounds__(32 * kNuWarps)
 nextuse_kernel(wf_dev_problem dp, wf_plans pl, const uint32_t *status, uint16_t *table)
 {
@@ -984,9 +992,9 @@ nextuse_kernel(wf_dev_problem dp, wf_plans pl, const uint32_t *status, uint16_t 
         uint16_t *out = table + p * (int64_t)N;
         for (int32_t k = lane; k < D * M; k += 32) last[k] = 0xFFFFu;
         __syncwarp();
-        // Three chunks of gathers are in flight ahead of the one being settled:
-        // its dispatch entries, then their nodes' placement, record and fusion
-        // word, then the placement of their fusible predecessors.
+        // The chunks ahead: dispatch entries, then their nodes' placement,
+        // record and fusion word, then the placement of their fusible
+        // predecessors.
         const int32_t top = ((N - 1) / 32) * 32 + lane;
         auto entry = [&](int32_t j) { return j >= 0 && j < N ? (int32_t)__ldg(order + j) : 0; };
         struct Node {
@@ -997,19 +1005,33 @@ nextuse_kernel(wf_dev_problem dp, wf_plans pl, const uint32_t *status, uint16_t 
             return Node{__ldg(place + h), (uint32_t)h, hr.x, (hr.y >> 16) & 15u, __ldg(fuse + (h >> 5))};
         };
         auto before = [&](const Node &n) { return (n.links & 0xFFFFu) != 0xFFFFu ? (uint32_t)__ldg(place + (n.links & 0xFFFFu)) : ~0u; };
-        Node n1 = node(entry(top)), n2 = node(entry(top - 32));
-        uint32_t p1 = before(n1);
-        int32_t h3 = entry(top - 64);
+        Node n1, n2;
+        uint32_t p1 = 0;
+        int32_t h3 = 0;
+        if constexpr (kDeep) {
+            n1 = node(entry(top));
+            n2 = node(entry(top - 32));
+            p1 = before(n1);
+            h3 = entry(top - 64);
+        }
         for (int32_t base = ((N - 1) / 32) * 32; base >= 0; base -= 32) {
             const int32_t j = base + lane;
-            const Node n = n1;
-            const uint32_t pn = p1;
-            n1 = n2;
-            p1 = before(n1);
-            n2 = node(h3);
-            h3 = entry(j - 96);
             uint32_t key = 0xFFFFFFFFu;  // not the start of a unit
-            if (j < N && !(((n.fw >> (n.x & 31)) & 1u) && pn == n.d)) key = n.d * M + n.model;
+            if constexpr (kDeep) {
+                const Node n = n1;
+                const uint32_t pn = p1;
+                n1 = n2;
+                p1 = before(n1);
+                n2 = node(h3);
+                h3 = entry(j - 96);
+                if (j < N && !(((n.fw >> (n.x & 31)) & 1u) && pn == n.d)) key = n.d * M + n.model;
+            } else if (j < N) {
+                const int32_t x = __ldg(order + j);
+                const uint32_t d = __ldg(place + x);
+                const uint4 hr = __ldg(dp.hrec + x);
+                const uint32_t fp = hr.x & 0xFFFFu;
+                if (fp == 0xFFFFu || !bit_of_g(fuse, x) || __ldg(place + fp) != d) key = d * M + ((hr.y >> 16) & 15u);
+            }
             const uint32_t same = __match_any_sync(0xFFFFFFFFu, key);
             const uint32_t above = lane == 31 ? 0u : (same & (0xFFFFFFFFu << (lane + 1)));
             if (key != 0xFFFFFFFFu) out[j] = above ? (uint16_t)(base + __ffs((int)above) - 1) : last[key];
@@ -1381,7 +1403,8 @@ int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, c
     const wf_dev_problem &dp = ctx->dp;
     const size_t smem = (size_t)kNuWarps * dp.D * dp.M * sizeof(uint16_t);
     const int64_t blocks = std::min<int64_t>((pl->P + kNuWarps - 1) / kNuWarps, (int64_t)ctx->sms * 16);
-    nextuse_kernel<<<(unsigned)blocks, 32 * kNuWarps, smem, st>>>(dp, *pl, out->status, dp.nextuse);
+    const auto k = dp.N > kNuShort ? nextuse_kernel<true> : nextuse_kernel<false>;
+    k<<<(unsigned)blocks, 32 * kNuWarps, smem, st>>>(dp, *pl, out->status, dp.nextuse);
     return wf_cuda_check(cudaGetLastError(), "next-use launch");
 }
 

@@ -98,7 +98,7 @@ def test_tied_and_nearly_tied_quotients(loads, D, M):
 
 
 @pytest.mark.parametrize("D,M,P,scale", [(1, 1, 5, 1), (4, 2, 333, 1), (3, 3, 200, 1), (9, 4, 100, 1), (32, 4, 33, 1), (3, 5, 100, 1),
-                                         (2, 4, 100, 150000), (4, 1, 100, 1 << 20)])
+                                         (2, 4, 100, 400000), (4, 1, 100, 1 << 20)])
 def test_few_models(D, M, P, scale):
     """Four lanes a plan up to four models (and five models on eight lanes),
     with retain rows, invalid plans and run times that leave 32 bits."""
@@ -109,6 +109,19 @@ def test_few_models(D, M, P, scale):
     if P > 8:
         plans.place[3, 1] = D
         plans.order[5, 0] = plans.order[5, 1]
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 63, 64, 65, 96, 97])
+def test_window_lengths_of_the_next_use_pass(n):
+    """One to four chunks of 32 positions: the pass without reads ahead (up to
+    64 activations) and with them, chains that fuse across chunks."""
+    from test_gpu_edges import chains_window
+    prob = chains_window([n - n // 2, n // 2] if n > 1 else [1], D=2, M=1, seed=n)
+    rng = np.random.default_rng(n)
+    prob = prob.with_(reclaim=1, M=3, model=np.sort(rng.integers(0, 3, n)).astype(np.uint8), weight_mib=np.array([2, 3, 4], np.int32),
+                      peak_mib=np.full(2 * n, 6, np.int32), load_us=rng.integers(1, 100, 6).astype(np.int32))
+    plans = wfgen.make_plans(prob, 150, n)
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
 
 
