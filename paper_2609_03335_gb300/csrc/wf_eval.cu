@@ -4,11 +4,13 @@
 // loads / prefetches on the consumer's device (Eq. 5, Eq. 9), retain /
 // reclaim and the metrics of Section 4.2-4.3.
 //
-// Mapping: one thread plays one (plan, sample).  Its mutable state (chain-tail
-// finish times, per-device and per-session state) lives in a scratch row of
-// the context; plans beyond the number of rows are taken in rounds.  For
-// wf_eval_plans_phi a deterministic play also returns the window terms of
-// Eq. 12's ranking key (timely prefetches, lifecycle overhead).
+// Mapping: a warp plays a deterministic plan (warp_play); for
+// wf_eval_plans_phi it also returns the window terms of Eq. 12's ranking key
+// (timely prefetches, lifecycle overhead).  One thread plays one (plan, sample)
+// of a stochastic window, or one plan under the replica batch limit: its
+// mutable state (chain-tail finish times, per-device and per-session state)
+// lives in a scratch row of the context, and plans beyond the number of rows
+// are taken in rounds.
 #include <algorithm>
 #include <mutex>
 
@@ -403,17 +405,19 @@ __device__ __forceinline__ int32_t p95_rank(int64_t n) { return (int32_t)((95 * 
 // times (108 warp instructions per plan-position), 0.57 ms on u32 times (80).
 // ---------------------------------------------------------------------------
 
-// The warp's working memory: B's answers for C [32], device free times [D],
-// finish times of unit tails [N] and one more entry that stays 0 (the
-// predecessor of a node without one), and the sessions' last finishes plus
-// one [W] (0 = none yet).
+// The warp's working memory: B's answers for C [32], the models' weights [16],
+// device free times [D], finish times of unit tails [N] and one more entry
+// that stays 0 (the predecessor of a node without one), and the sessions' last
+// finishes [W].  Times count from 1, so that 0 is none yet.
 template <typename TT>
 struct WarpMem {
     uint2 *res;
+    int32_t *weight;
     TT *tfree, *ctail, *comp;
 };
 
-__host__ __device__ inline size_t warp_small_bytes(int32_t D) { return 32 * sizeof(uint2) + 8 * (size_t)D; }
+constexpr size_t kWarpHead = 32 * sizeof(uint2) + 16 * sizeof(int32_t);
+__host__ __device__ inline size_t warp_small_bytes(int32_t D) { return kWarpHead + 8 * (size_t)D; }
 template <typename TT>
 __host__ __device__ inline size_t warp_full_bytes(const wf_dev_problem &dp)
 {
@@ -427,7 +431,8 @@ __device__ __forceinline__ WarpMem<TT> warp_mem(const wf_dev_problem &dp, uint8_
 {
     WarpMem<TT> w;
     w.res = (uint2 *)sm;
-    w.tfree = (TT *)(sm + 32 * sizeof(uint2));
+    w.weight = (int32_t *)(sm + 32 * sizeof(uint2));
+    w.tfree = (TT *)(sm + kWarpHead);
     w.ctail = (TT *)big;
     w.comp = w.ctail + dp.N + 1;
     return w;
@@ -493,11 +498,10 @@ __device__ __forceinline__ int64_t warp_sum(int64_t v)
     return v;
 }
 
-__device__ __forceinline__ int64_t warp_max(int64_t v)
+__device__ __forceinline__ uint64_t warp_max(uint64_t v)
 {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
+    const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(v >> 32));
+    return ((uint64_t)hi << 32) | __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
 }
 
 struct PlayResult {
@@ -506,9 +510,10 @@ struct PlayResult {
 
 // One play of a valid plan; every lane returns the results (mk still counts
 // from 0, not from the first arrival).  kPhi adds the window terms of Eq. 12;
-// Q is the residency queue's word.  With u32 times, false when some time
+// Q is the residency queue's word; kShort walks step C over the lanes that
+// start a unit instead of over all 32, unrolled.  With u32 times, false when some time
 // leaves 32 bits (the results are then void).
-template <typename TT, typename Q, bool kPhi>
+template <typename TT, typename Q, bool kPhi, bool kShort>
 __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const WarpMem<TT> &wm, PlayResult &r)
 {
     constexpr bool kNarrow = sizeof(TT) == 4;
@@ -517,11 +522,11 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
     for (int32_t w = lane; w < W; w += 32) wm.comp[w] = 0;
     for (int32_t d = lane; d < D; d += 32) wm.tfree[d] = 0;
     if (lane == 0) wm.ctail[N] = 0;
-    // The lane's device: queue, resident count and weights, models ever held.
-    Q queue = 0;
-    uint32_t nres = 0, used = 0, ever = 0;
-    const uint32_t capd = lane < D ? (uint32_t)__ldg(dp.cap + lane) : 0u;
-    TT end = 0;
+    if (lane < 16) wm.weight[lane] = lane < dp.M ? __ldg(dp.weight + lane) : 0;
+    // The lane's device, and the models it ever held.
+    DevState<Q> ds;
+    ds.init(lane < D ? (uint32_t)__ldg(dp.cap + lane) : 0u);
+    uint32_t ever = 0;
     int64_t gsum = 0, timely = 0, life = 0;
     bool ovf = false;
     __syncwarp();
@@ -546,8 +551,8 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
                 kv = max(kv, __ldg(dp.peak + (int64_t)s * D + d) - wgt);
                 tail = s;
             }
-        const TT arr = (TT)arr64, run = (TT)run64;
-        if (kNarrow) ovf |= unit && ((arr64 | run64) >> 32) != 0;
+        const TT arr = (TT)(arr64 + 1), run = (TT)run64;
+        if (kNarrow) ovf |= unit && (((arr64 + 1) | run64) >> 32) != 0;
         const bool drop = unit && pr.retain && !bit_at(pr.retain, tail);
         const uint32_t w3 = (uint32_t)d | ((uint32_t)m << 5) | (pf ? kPrefetch : 0u) | (drop ? kDrop : 0u);
         // B: residency of the chunk's units on the lane's device.
@@ -561,7 +566,7 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
             const uint32_t r1 = __shfl_sync(0xFFFFFFFFu, (uint32_t)kv, k), r3 = __shfl_sync(0xFFFFFFFFu, w3, k);
             if (mine) {
                 bool missed;
-                uint2 x = settle_lru<Q>(queue, nres, used, capd, r1, r3, dp.weight, dp.load, D, dp.err, missed);
+                uint2 x = ds.settle(r1, r3, wm.weight, dp.load, D, dp.err, missed);
                 if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
                     const uint32_t mk = (r3 >> 5) & 15u;
                     x.x |= ((ever >> mk) & 1u) << 31;
@@ -576,20 +581,20 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
         const uint2 x = wm.res[lane];
         const TT ld = kPhi ? x.x & 0x7FFFFFFFu : x.x;
         const int turn = unit ? lane : 32;
-#pragma unroll 4
-        for (int k = 0; k < 32; ++k) {
+        TT *const tfree = wm.tfree + d, *const done = wm.ctail + tail, *const comp = wm.comp + w;
+        const TT *const pred0 = wm.ctail + p0, *const pred1 = wm.ctail + p1;
+        const auto play_unit = [&](int k) {
             if (turn == k) {
-                const TT tf = wm.tfree[d];
-                TT rel = max(arr, max(wm.ctail[p0], wm.ctail[p1]));  // Eq. 2, Eq. 7
+                const TT tf = *tfree;
+                TT rel = max(arr, max(*pred0, *pred1));  // Eq. 2, Eq. 7
                 for (int32_t e = 2; e < np; ++e) rel = max(rel, wm.ctail[__ldg(dp.pred_idx + e0 + e)]);
                 // (on a hit the load time is 0 and the prefetch bit cleared)
                 const TT ls = max(tf, (x.y & kPrefetch) ? arr : rel), le = ls + ld;
                 const TT start = max(le, rel), c = start + run;
                 if (kNarrow) ovf |= le < ls || c < start;
-                wm.ctail[tail] = c;
-                wm.tfree[d] = c;
-                wm.comp[w] = max(wm.comp[w], c + 1);
-                end = max(end, c);
+                *done = c;
+                *tfree = c;
+                *comp = max(*comp, c);
                 if (x.y & (kWasEmpty | kEmptied)) {
                     if (x.y & kWasEmpty) gsum -= (int64_t)ls;
                     if (x.y & kEmptied) gsum += (int64_t)c;
@@ -600,16 +605,24 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
                 }
             }
             __syncwarp();
+        };
+        if constexpr (kShort) {
+#pragma unroll 1
+            for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, unit); todo; todo &= todo - 1) play_unit(__ffs((int)todo) - 1);
+        } else {
+#pragma unroll 4
+            for (int k = 0; k < 32; ++k) play_unit(k);
         }
         if (kNarrow && __any_sync(0xFFFFFFFFu, ovf)) return false;
     }
-    const int64_t open = __popc(__ballot_sync(0xFFFFFFFFu, lane < D && nres != 0));  // devices occupied to the end
-    r.mk = warp_max((int64_t)end);
-    if (kNarrow && r.mk == 0xFFFFFFFFll) return false;  // (one plus it has wrapped)
-    r.gpu = warp_sum(gsum) + open * r.mk;
+    const int64_t open = __popc(__ballot_sync(0xFFFFFFFFu, lane < D && ds.occupied()));  // devices occupied to the end
+    const int64_t end = (int64_t)warp_max(lane < D ? wm.tfree[lane] : (TT)0);
+    r.mk = end - 1;
+    r.gpu = warp_sum(gsum) + open * end;
     r.timely = kPhi ? warp_sum(timely) : 0;
     r.life = kPhi ? warp_sum(life) : 0;
-    r.p95 = (int64_t)(warp_select(LatencyArr<TT>{wm.comp, dp.arrival}, W, p95_rank(W)) ^ (1ull << 63));
+    const LatencyArr<TT> lat{wm.comp, dp.arrival};
+    r.p95 = (int64_t)((W <= 32 ? warp_select<1>(lat, W, p95_rank(W)) : warp_select<8>(lat, W, p95_rank(W))) ^ (1ull << 63));
     __syncwarp();  // the memory is free for the next plan
     return true;
 }
@@ -631,28 +644,57 @@ __device__ __forceinline__ void put_result(const wf_dev_problem &dp, const wf_ev
 
 constexpr size_t kSmemMax = 227 * 1024;
 
+// How the warps that play a plan each are launched.
+//   kFour  four warps a CTA on 64 registers, so that 32 plans are resident on
+//          an SM; step C only over the lanes that start a unit
+//   kSolo  a warp a CTA, finish times in shared memory
+//   kRows  a warp a CTA, finish times in a row of global scratch (windows that
+//          exceed shared memory)
+enum WarpShape { kFour, kSolo, kRows };
+__host__ __device__ constexpr int warps_of(WarpShape s) { return s == kFour ? 4 : 1; }
+constexpr int kSolo64 = 12, kSolo32 = 16;  // CTAs of kSolo that registers allow an SM, on u64 and on u32 times
+
+// Shared memory of a warp.
+template <typename TT>
+__host__ __device__ inline size_t warp_bytes(const wf_dev_problem &dp, WarpShape s)
+{
+    return ((s == kRows ? warp_small_bytes(dp.D) : warp_full_bytes<TT>(dp)) + 15) & ~(size_t)15;
+}
+
+// The shape for P plans of a window whose warps take `bytes` each with finish
+// times in shared memory:
+//   kFour where 32 such warps fit an SM and there are more plans than kSolo
+//   holds at once.  Short windows in large batches are bound by issue, a CTA of
+//   one warp at a time leaves its registers' share of the SM idle: 40,000 plans of N =
+//   14, D = 7, M = 12 in wf_eval_plans_static, us: a thread per plan 142, kSolo
+//   153, kFour 101; 65,536 of N = 40 on the int64 path 319, 452, 314; 3,700 of
+//   N = 1,000 in the static call 7,385, 535, 426.
+WarpShape warp_shape(int sms, int64_t P, size_t bytes)
+{
+    if (bytes > kSmemMax) return kRows;
+    if (32 * bytes <= kSmemMax && P > kSolo32 * (int64_t)sms) return kFour;
+    return kSolo;
+}
+
 // Every plan of the batch, or (list) the plans whose times a sweep could not
-// hold, on int64 times; a CTA is one warp and walks over plans.  Finish times
-// in shared memory (kShared), else in a row of the context's scratch (windows
-// beyond about 28,000 activations).
-template <bool kShared>
-__global__ void __launch_bounds__(32, 12)
+// hold, on int64 times; a warp walks over plans.
+template <typename Q, bool kPhi, WarpShape kShape>
+__global__ void __launch_bounds__(32 * warps_of(kShape), kShape == kFour ? 8 : kSolo64)
 eval_warp_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
                  const int32_t *list, const int32_t *count)
 {
     extern __shared__ __align__(16) uint8_t esm[];
-    const int64_t n = list ? (int64_t)*count : pl.P;
-    uint8_t *big = kShared ? esm + warp_small_bytes(dp.D) : scratch + (size_t)blockIdx.x * row_bytes;
-    const WarpMem<uint64_t> wm = warp_mem<uint64_t>(dp, esm, big);
-    for (int64_t k = blockIdx.x; k < n; k += gridDim.x) {
+    constexpr int kW = warps_of(kShape);
+    const int64_t n = list ? (int64_t)*count : pl.P, k0 = (int64_t)blockIdx.x * kW + (threadIdx.x >> 5);
+    uint8_t *sm = esm + (threadIdx.x >> 5) * warp_bytes<uint64_t>(dp, kShape);
+    uint8_t *big = kShape == kRows ? scratch + (size_t)k0 * row_bytes : sm + warp_small_bytes(dp.D);
+    const WarpMem<uint64_t> wm = warp_mem<uint64_t>(dp, sm, big);
+    for (int64_t k = k0; k < n; k += (int64_t)gridDim.x * kW) {
         const int64_t p = list ? (int64_t)list[k] : k;
         const PlanRows pr = plan_rows(pl, p);
         const uint32_t st = warp_status(dp, pr, (uint16_t *)big);
         PlayResult r = {};
-        if (!st) {
-            if (dp.phi_life) warp_play<uint64_t, uint64_t, true>(dp, pr, wm, r);
-            else warp_play<uint64_t, uint64_t, false>(dp, pr, wm, r);
-        }
+        if (!st) warp_play<uint64_t, Q, kPhi, kShape == kFour>(dp, pr, wm, r);
         put_result(dp, out, p, st, r, dp.first_arrival);
     }
 }
@@ -802,18 +844,28 @@ int launch_int64(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, con
         eval_batched_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes,
                                                                       units, list, count);
     } else {
-        const bool shared = warp_full_bytes<uint64_t>(dp) <= kSmemMax;
-        const size_t smem = shared ? warp_full_bytes<uint64_t>(dp) : warp_small_bytes(dp.D);
-        const auto kernel = shared ? eval_warp_kernel<true> : eval_warp_kernel<false>;
+        const size_t bytes = warp_bytes<uint64_t>(dp, kSolo);
+        // A list is most often empty: few CTAs where that can be.
+        const WarpShape shape = list && 32 * bytes <= kSmemMax ? kFour : warp_shape(ctx->sms, plans->P, bytes);
+        const size_t smem = warps_of(shape) * warp_bytes<uint64_t>(dp, shape);
+        const auto by_phi = [&](auto q, auto s) {
+            using Q = typename decltype(q)::type;
+            constexpr WarpShape kS = (WarpShape)decltype(s)::value;
+            return dp.phi_life ? eval_warp_kernel<Q, true, kS> : eval_warp_kernel<Q, false, kS>;
+        };
+        const auto by_shape = [&](auto q) {
+            return shape == kFour ? by_phi(q, Iv<kFour>{}) : shape == kSolo ? by_phi(q, Iv<kSolo>{}) : by_phi(q, Iv<kRows>{});
+        };
+        const auto kernel = dp.M <= 8 ? by_shape(Ty<uint32_t>{}) : by_shape(Ty<uint64_t>{});
         const int rc = wf_cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                           (int)smem), "int64 path smem attribute");
         if (rc) return rc;
-        // A CTA per plan, or (a list, most often empty) about as many as fit
-        // the chip at once; beyond shared memory, a scratch row per CTA.
-        int64_t blocks = plans->P;
-        if (list) blocks = std::min<int64_t>(blocks, (int64_t)ctx->sms * 12);
-        if (!shared) blocks = std::min<int64_t>(blocks, units);
-        kernel<<<(unsigned)blocks, 32, smem, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes, list, count);
+        // A warp per plan, or for a list about as many as fit the chip at
+        // once; with rows, a row per CTA.
+        int64_t blocks = (plans->P + warps_of(shape) - 1) / warps_of(shape);
+        if (list) blocks = std::min<int64_t>(blocks, (int64_t)ctx->sms * (kSolo64 / warps_of(shape)));
+        if (shape == kRows) blocks = std::min<int64_t>(blocks, units);
+        kernel<<<(unsigned)blocks, 32 * warps_of(shape), smem, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes, list, count);
     }
     return wf_cuda_check(cudaGetLastError(), "int64 pass launch");
 }
@@ -1034,30 +1086,33 @@ __global__ void static_link_kernel(uint8_t *s, wf_dev_problem dp, StaticLayout l
     }
 }
 
-// The deterministic evaluation, a warp (a CTA) per plan, with the first
-// arrival taken from the static header: on u32 times in shared memory
-// (kShared), and on u64 times in the plan's scratch row when those do not
-// hold the plan or the window does not fit.
-template <typename Q, bool kShared>
-__global__ void __launch_bounds__(32, 16)
+// The deterministic evaluation, a warp per plan, with the first
+// arrival taken from the static header: on u32 times in shared memory, and
+// on u64 times in the plan's scratch row when those do not hold the plan or
+// the window does not fit (kRows).
+template <typename Q, WarpShape kShape>
+__global__ void __launch_bounds__(32 * warps_of(kShape), kShape == kFour ? 8 : kSolo32)
 eval_static_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *s, StaticLayout l,
                    size_t row_bytes)
 {
     extern __shared__ __align__(16) uint8_t esm[];
-    const int64_t p = blockIdx.x;
+    const int64_t p = (int64_t)blockIdx.x * warps_of(kShape) + (threadIdx.x >> 5);
+    if (p >= pl.P) return;  // the whole warp
     if ((*(volatile int *)(s + 8) & 0xFF) == kStaticBadTables) {  // nothing is evaluated
-        if (threadIdx.x == 0) {
+        if ((threadIdx.x & 31) == 0) {
             out.status[p] = WF_ST_TABLES;
             out.makespan_us[p] = out.p95_us[p] = out.gpu_us[p] = WF_INF64;
         }
         return;
     }
-    uint8_t *row = s + l.rows + (size_t)p * row_bytes, *big = kShared ? esm + warp_small_bytes(dp.D) : row;
+    uint8_t *sm = esm + (threadIdx.x >> 5) * warp_bytes<uint32_t>(dp, kShape);
+    uint8_t *row = s + l.rows + (size_t)p * row_bytes, *big = kShape == kRows ? row : sm + warp_small_bytes(dp.D);
     const PlanRows pr = plan_rows(pl, p);
     const uint32_t st = warp_status(dp, pr, (uint16_t *)big);
     PlayResult r = {};
-    if (!st && !(kShared && warp_play<uint32_t, Q, false>(dp, pr, warp_mem<uint32_t>(dp, esm, big), r)))
-        warp_play<uint64_t, Q, false>(dp, pr, warp_mem<uint64_t>(dp, esm, row), r);
+    constexpr bool kShort = kShape == kFour;
+    if (!st && !(kShape != kRows && warp_play<uint32_t, Q, false, kShort>(dp, pr, warp_mem<uint32_t>(dp, sm, big), r)))
+        warp_play<uint64_t, Q, false, kShort>(dp, pr, warp_mem<uint64_t>(dp, sm, row), r);
     put_result(dp, out, p, st, r, *(const int64_t *)s);
 }
 
@@ -1153,14 +1208,21 @@ extern "C" int wf_eval_plans_static(const wf_problem *pb, const wf_plans *pl, co
     static_check_kernel<<<(unsigned)((cspan + 255) / 256), 256, 0, st>>>(s, dp);
     static_count_kernel<<<grid, 256, 0, st>>>(s, dp, l);
     static_link_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(s, dp, l);
-    const bool shared = warp_full_bytes<uint32_t>(dp) <= kSmemMax;
-    const size_t smem = shared ? warp_full_bytes<uint32_t>(dp) : warp_small_bytes(D);
-    const auto kernel = M <= 8 ? (shared ? eval_static_kernel<uint32_t, true> : eval_static_kernel<uint32_t, false>)
-                               : (shared ? eval_static_kernel<uint64_t, true> : eval_static_kernel<uint64_t, false>);
+    int sms = 0;
+    rc = wf_cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    if (rc) return rc;
+    const WarpShape shape = warp_shape(sms, pl->P, warp_bytes<uint32_t>(dp, kSolo));
+    const size_t smem = warps_of(shape) * warp_bytes<uint32_t>(dp, shape);
+    const auto by_shape = [&](auto q) {
+        using Q = typename decltype(q)::type;
+        return shape == kFour ? eval_static_kernel<Q, kFour> : shape == kSolo ? eval_static_kernel<Q, kSolo> : eval_static_kernel<Q, kRows>;
+    };
+    const auto kernel = M <= 8 ? by_shape(Ty<uint32_t>{}) : by_shape(Ty<uint64_t>{});
     rc = wf_cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                        "static evaluation smem attribute");
     if (rc) return rc;
-    kernel<<<(unsigned)pl->P, 32, smem, st>>>(dp, *pl, *out, s, l, row);
+    const unsigned blocks = (unsigned)((pl->P + warps_of(shape) - 1) / warps_of(shape));
+    kernel<<<blocks, 32 * warps_of(shape), smem, st>>>(dp, *pl, *out, s, l, row);
     return wf_cuda_check(cudaGetLastError(), "static evaluation launch");
 }
 

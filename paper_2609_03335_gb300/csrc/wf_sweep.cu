@@ -150,118 +150,6 @@ struct PairArr {
     }
 };
 
-// Residency of one device under least-recently-used reclamation in one
-// shared-memory word: the queue of 4-bit model ids, least recently used in
-// nibble 0, empty places 0xF, and the free capacity (capacity minus resident
-// weights); up to 8 models the queue says its own length (no id has bit 3
-// set), beyond it is kept beside.  settle() plays a unit's admission (Eq. 11,
-// Section 3.5): the unit's own model leaves the queue first, the victims are
-// then its first entries, and the model goes back in last.  The first three
-// victims' weights are read at once and taken without branching (a loop over
-// victims waited for one weight at a time: about 130 instructions a unit with
-// it, half of that without).  Returns the record's rewritten (w1, w3): the
-// load the unit waits for (none on a hit, Eq. 5) and the occupancy changes.
-template <typename Q>
-struct DevState;
-
-// The victims: from `need` and the free capacity f, the shift that drops the
-// evicted entries from queue q (at most n4 / 4 of them).
-template <typename Q>
-__device__ __forceinline__ int evict(Q q, uint32_t need, uint32_t &f, int n4, const int32_t *weight)
-{
-    const uint32_t w0 = (uint32_t)weight[(uint32_t)q & 15u], w1 = (uint32_t)weight[(uint32_t)(q >> 4) & 15u],
-                   w2 = (uint32_t)weight[(uint32_t)(q >> 8) & 15u];
-    int e4 = 0;
-    if (need > f) { f += w0; e4 = 4; }
-    if (need > f) { f += w1; e4 = 8; }
-    if (need > f) { f += w2; e4 = 12; }
-    for (; need > f && e4 < n4; e4 += 4) f += (uint32_t)weight[(uint32_t)(q >> e4) & 15u];
-    return min(e4, n4);
-}
-
-__device__ __forceinline__ uint2 settled(uint32_t r3, bool hit, uint32_t ld, bool was_empty, bool emptied)
-{
-    return make_uint2(hit ? 0u : ld, (r3 & ~(hit ? kPrefetch | kWasEmpty : kWasEmpty)) | (was_empty ? kWasEmpty : 0u) |
-                                         (emptied ? kEmptied : 0u));
-}
-
-template <>
-struct DevState<uint32_t> {
-    uint2 v;  // queue, free capacity
-    __device__ __forceinline__ void init(uint32_t cap) { v = make_uint2(~0u, cap); }
-    __device__ __forceinline__ bool occupied() const { return v.x != ~0u; }
-    __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
-                                            int32_t D, int *err, bool &missed)
-    {
-        const uint32_t m = (r3 >> 5) & 15u, wm = (uint32_t)weight[m], ld = (uint32_t)load[m * D + (r3 & 31u)];
-        uint32_t q = v.x, f = v.y;
-        const bool was_empty = q == ~0u;
-        const uint32_t x = q ^ (0x11111111u * m);
-        const uint32_t z = (x - 0x11111111u) & ~x & 0x88888888u;  // its lowest bit: the nibble equal to m
-        const bool hit = z != 0;
-        missed = !hit;
-        const uint32_t below = ((z & (0u - z)) >> 3) - 1u;  // the bits below that nibble (all when there is none)
-        q = (q & below) | ((q >> 4) & ~below) | 0xF0000000u;
-        const uint32_t need = hit ? r1 : wm + r1;  // at most the capacity
-        const int e4 = evict(q, need, f, 32, weight);
-        if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
-        q = __funnelshift_rc(q, ~0u, e4);
-        const uint32_t gap = q & 0x88888888u;
-        const uint32_t at = (gap & (0u - gap)) >> 3;  // 1 << 4 n: the first empty place
-        const uint32_t with = q - (15u - m) * at;     // 0xF there becomes m
-        f -= hit ? 0u : wm;
-        bool emptied = false;
-        if (r3 & kDrop) {  // the model leaves when the unit ends
-            f += wm;
-            emptied = q == ~0u;
-        } else {
-            q = with;
-        }
-        v = make_uint2(q, f);
-        return settled(r3, hit, ld, was_empty, emptied);
-    }
-};
-
-template <>
-struct DevState<uint64_t> {
-    uint4 v;  // queue (low, high), free capacity, models held
-    __device__ __forceinline__ void init(uint32_t cap) { v = make_uint4(~0u, ~0u, cap, 0u); }
-    __device__ __forceinline__ bool occupied() const { return v.w != 0; }
-    __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
-                                            int32_t D, int *err, bool &missed)
-    {
-        const uint32_t m = (r3 >> 5) & 15u, wm = (uint32_t)weight[m], ld = (uint32_t)load[m * D + (r3 & 31u)];
-        uint64_t q = ((uint64_t)v.y << 32) | v.x;
-        uint32_t f = v.z, n = v.w;
-        const bool was_empty = n == 0;
-        const uint64_t x = q ^ (0x1111111111111111ull * m);
-        const uint64_t z = (x - 0x1111111111111111ull) & ~x & 0x8888888888888888ull;
-        const uint64_t low = (z & (0ull - z)) >> 3;
-        // (with 16 models the empty places match the last one)
-        const bool hit = low != 0 && (uint32_t)__popcll(low - 1) < 4 * n;
-        missed = !hit;
-        const uint64_t below = hit ? low - 1 : ~0ull;
-        q = (q & below) | ((q >> 4) & ~below) | (hit ? 0xFull << 60 : 0ull);
-        n -= hit ? 1u : 0u;
-        const uint32_t need = hit ? r1 : wm + r1;
-        const int e4 = evict(q, need, f, (int)(4 * n), weight);
-        if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
-        q = e4 < 64 ? (q >> e4) | ~(~0ull >> e4) : ~0ull;
-        n -= (uint32_t)e4 >> 2;
-        f -= hit ? 0u : wm;
-        bool emptied = false;
-        if (r3 & kDrop) {
-            f += wm;
-            emptied = n == 0;
-        } else {
-            q ^= (uint64_t)(15u ^ m) << (4 * n);
-            n += 1;
-        }
-        v = make_uint4((uint32_t)q, (uint32_t)(q >> 32), f, n);
-        return settled(r3, hit, ld, was_empty, emptied);
-    }
-};
-
 struct PcLayout {
     uint32_t weight, load, rcost, wsum, arr, ring, next, slots, slots_hi, tfree, free, queue, open, flag, gmask, everl, total;
 };

@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import wfgen
-from gpu_util import THREADS, lib
+from gpu_util import THREADS, gpu_eval, lib
 from randprob import random_problem
 from test_gpu_parity import inject_invalid
 
@@ -106,3 +106,19 @@ def test_large_topk_and_stochastic_refusal():
     t = torch.empty(8, dtype=torch.int64, device="cuda")
     with pytest.raises(wf.WfError):
         wf.wf_eval_plans_phi(ctx, dp, wf.Results(8), t, torch.empty_like(t))
+
+
+@pytest.mark.parametrize("D,M,more", [(3, 4, 3), (12, 11, 0), (32, 16, 1), (1, 1, 2)])
+def test_int64_path_on_large_batches_of_short_windows(D, M, more):
+    """More plans than 16 an SM, four warps a CTA, the last CTA full and not:
+    with the window terms, and without them on the same plans."""
+    import torch
+    P = 16 * torch.cuda.get_device_properties(0).multi_processor_count + 1 + more
+    rng = np.random.default_rng(60 + D)
+    prob = random_problem(rng, n_sessions=5, sizes=(4, 11), D=D, M=M)
+    plans = wfgen.make_plans(prob, P, D, p_retain=0.7 if D > 3 else None)
+    inject_invalid(plans, prob, rng)
+    got = check(prob, plans, k=16, int64_path=True)
+    plain = gpu_eval(prob, plans, int64_path=True)
+    for name in ("makespan", "p95", "gpu", "status"):
+        assert np.array_equal(got[name], plain[name])

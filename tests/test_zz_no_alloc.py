@@ -164,6 +164,32 @@ def test_static_entry_on_edges(sessions, sizes, D, M, scale):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("D,M,scale", [(3, 4, 1), (7, 12, 1), (32, 16, 1), (2, 3, 1 << 20)])
+def test_large_batches_of_short_windows(D, M, scale):
+    """Batches around the one from which four warps share a CTA (16 plans an
+    SM), the last CTA full and not, with and without retain rows, some invalid
+    plans, and (the largest scale) run times that leave 32 bits."""
+    import torch
+    from randprob import random_problem
+    from paper_2609_03335_gb300 import build, wf
+    build.build()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(40 + D)
+    prob = random_problem(rng, n_sessions=4, sizes=(4, 12), D=D, M=M)
+    prob = prob.with_(lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, 2**31 - 1).astype(np.int32))
+    plans = wfgen.make_plans(prob, 16 * sms + 6, 5, p_retain=0.7 if D % 2 else None)
+    plans.place[2, 0] = prob.D
+    plans.order[4, 0] = plans.order[4, 1]
+    want = oracle.eval_plans(prob, plans)
+    dprob = wf.DeviceProblem(prob)
+    for P in (16 * sms + 6, 16 * sms + 1, 16 * sms):
+        out = wf.Results(P)
+        wf.wf_eval_plans_static(dprob, wf.DevicePlans.from_host(plans.slice(0, P), "cuda"), out)
+        wf.wf_static_status()
+        for a, b in zip(out.numpy(), want):
+            assert np.array_equal(a, b[:P])
+
+
 @pytest.mark.parametrize("others", [[1] * 19, [1] * 3 + [0] * 16, [0] * 19, [3, 2, 1, 1, 0, 0], [1] * 250 + [2] * 60 + [0] * 5,
                                     [1] * 900 + [0] * 200])
 def test_static_entry_with_sessions_that_own_no_activation(others):
