@@ -648,8 +648,8 @@ constexpr size_t kSmemMax = 227 * 1024;
 //   kFour  four warps a CTA on 64 registers, so that 32 plans are resident on
 //          an SM; step C only over the lanes that start a unit
 //   kSolo  a warp a CTA, finish times in shared memory
-//   kRows  a warp a CTA, finish times in a row of global scratch (windows that
-//          exceed shared memory)
+//   kRows  a warp a CTA, finish times in a row of global scratch, which L2
+//          holds for the most part
 enum WarpShape { kFour, kSolo, kRows };
 __host__ __device__ constexpr int warps_of(WarpShape s) { return s == kFour ? 4 : 1; }
 constexpr int kSolo64 = 12, kSolo32 = 16;  // CTAs of kSolo that registers allow an SM, on u64 and on u32 times
@@ -662,18 +662,24 @@ __host__ __device__ inline size_t warp_bytes(const wf_dev_problem &dp, WarpShape
 }
 
 // The shape for P plans of a window whose warps take `bytes` each with finish
-// times in shared memory:
+// times in shared memory; solo: the most CTAs of kSolo an SM holds.
 //   kFour where 32 such warps fit an SM and there are more plans than kSolo
 //   holds at once.  Short windows in large batches are bound by issue, a CTA of
 //   one warp at a time leaves its registers' share of the SM idle: 40,000 plans of N =
 //   14, D = 7, M = 12 in wf_eval_plans_static, us: a thread per plan 142, kSolo
 //   153, kFour 101; 65,536 of N = 40 on the int64 path 319, 452, 314; 3,700 of
 //   N = 1,000 in the static call 7,385, 535, 426.
-WarpShape warp_shape(int sms, int64_t P, size_t bytes)
+//   kRows where shared memory holds fewer warps than registers do, once the
+//   plans exceed those (and where it holds none).  On the int64 path, ms in
+//   shared memory and in rows: N = 8,192, 256 plans 1.90 and 2.21, 4,096 plans 17.2 and
+//   6.60; N = 20,000, 152 plans (one an SM) 4.46 and 4.62, 512 plans 17.1 and
+//   4.75, 4,096 plans 119 and 12.6 (a thread per plan: 134).
+WarpShape warp_shape(int sms, int64_t P, size_t bytes, int solo)
 {
     if (bytes > kSmemMax) return kRows;
     if (32 * bytes <= kSmemMax && P > kSolo32 * (int64_t)sms) return kFour;
-    return kSolo;
+    const int64_t fit = (int64_t)(kSmemMax / bytes);
+    return fit < solo && P > fit * sms ? kRows : kSolo;
 }
 
 // Every plan of the batch, or (list) the plans whose times a sweep could not
@@ -846,7 +852,7 @@ int launch_int64(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, con
     } else {
         const size_t bytes = warp_bytes<uint64_t>(dp, kSolo);
         // A list is most often empty: few CTAs where that can be.
-        const WarpShape shape = list && 32 * bytes <= kSmemMax ? kFour : warp_shape(ctx->sms, plans->P, bytes);
+        const WarpShape shape = list && 32 * bytes <= kSmemMax ? kFour : warp_shape(ctx->sms, plans->P, bytes, kSolo64);
         const size_t smem = warps_of(shape) * warp_bytes<uint64_t>(dp, shape);
         const auto by_phi = [&](auto q, auto s) {
             using Q = typename decltype(q)::type;
@@ -1211,7 +1217,7 @@ extern "C" int wf_eval_plans_static(const wf_problem *pb, const wf_plans *pl, co
     int sms = 0;
     rc = wf_cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
     if (rc) return rc;
-    const WarpShape shape = warp_shape(sms, pl->P, warp_bytes<uint32_t>(dp, kSolo));
+    const WarpShape shape = warp_shape(sms, pl->P, warp_bytes<uint32_t>(dp, kSolo), kSolo32);
     const size_t smem = warps_of(shape) * warp_bytes<uint32_t>(dp, shape);
     const auto by_shape = [&](auto q) {
         using Q = typename decltype(q)::type;

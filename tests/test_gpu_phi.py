@@ -122,3 +122,21 @@ def test_int64_path_on_large_batches_of_short_windows(D, M, more):
     plain = gpu_eval(prob, plans, int64_path=True)
     for name in ("makespan", "p95", "gpu", "status"):
         assert np.array_equal(got[name], plain[name])
+
+
+@pytest.mark.parametrize("n,M,more", [(14500, 2, 1), (14500, 9, 1), (14500, 2, 0), (3000, 9, 9)])
+def test_int64_path_on_long_windows(n, M, more):
+    """Windows of which shared memory holds one plan an SM (or nine): as many
+    plans as it holds at once, and more, whose finish times lie in scratch rows."""
+    import torch
+    from test_gpu_edges import chains_window
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    P = sms * (1 if n > 10000 else 9) + more
+    prob = chains_window([n // 50] * 50, D=3, M=M, seed=M)
+    plans = wfgen.make_plans(prob, P, 2, p_retain=0.7 if M == 9 else None)
+    rng = np.random.default_rng(M)
+    inject_invalid(plans, prob, rng)
+    got = check(prob, plans, k=16, int64_path=True)
+    plain = gpu_eval(prob, plans, int64_path=True)
+    for name in ("makespan", "p95", "gpu", "status"):
+        assert np.array_equal(got[name], plain[name])
