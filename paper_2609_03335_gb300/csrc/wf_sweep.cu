@@ -11,7 +11,7 @@
 //   - finish-time slots (u32 microseconds) assigned statically from the DAG
 //     (wf_slots.cpp) instead of one word per activation, [slot][plan];
 //   - per device: free time [device][plan]; resident weights, count and LRU
-//     queue [device row][residency lane].
+//     queue [device][plan].
 // Status bits (Eq. 8-10) come first from status_kernel, a warp per plan.
 //
 // Times: the deterministic sweep first plays u32 times and lists a plan whose
@@ -92,17 +92,15 @@ struct PcShape {
 };
 
 // Residency lanes per plan under least-recently-used reclamation: a device
-// group each (d = g mod kG).  A lane's state for its t-th device (d = g + t kG)
-// sits at [t][lane]: the lanes of a warp touch consecutive words.  Under
+// group each (d = g mod kG), with a state per [device][plan].  Under
 // reclamation by next use the lanes are a plan's models, every device is
 // played by all of them (one group), and the state is [device][lane].
 template <int kP, int kReclaim, typename Q>
 struct PcGroups {
     using S = PcShape<kP, kReclaim, Q>;
     static constexpr int kG = kReclaim ? 1 : (32 * S::kRes) / kP;
-    static constexpr int kLanes = 32 * S::kRes;  // row length of the state
+    static constexpr int kRow = kReclaim ? 32 * S::kRes : kP;  // row length of the state
     static_assert(kG >= 1 && kG * kP <= 32 * S::kRes, "residency lanes");
-    __host__ __device__ static int32_t rows(int32_t D) { return (D + kG - 1) / kG; }
 };
 
 // Relative 32-bit times (slot storage Rel32, with TT = uint32_t): every time
@@ -158,8 +156,8 @@ struct PcLayout {
 // with reclamation by next use (kReclaim) the next uses lie beside the ring
 // and each plan keeps per (device, model) the next use and the last use
 // of the resident copy, and per device the free capacity; with the window
-// terms of Eq. 12 (kPhi) each residency lane keeps per device the models it
-// ever held (by next use: in a register, per model the devices).
+// terms of Eq. 12 (kPhi) each plan keeps per device the models it ever
+// held (by next use: in a register, per model the devices).
 template <int kP, typename TT, typename Q, int kReclaim = 0, bool kPhi = false, typename ST = TT>
 __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W, int32_t NS)
 {
@@ -177,15 +175,15 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
     l.slots = o; o += round16(SlotBytes<ST>::kLo * (uint32_t)NS * kP);
     l.slots_hi = o; o += round16(SlotBytes<ST>::kHi * (uint32_t)NS * kP);
     l.tfree = o; o += round16(t * D * kP);
-    const uint32_t rs = (uint32_t)(G::rows(D) * G::kLanes);
+    const uint32_t rs = (uint32_t)(D * G::kRow);
     // Residency state: a word per device (DevState), or under reclamation by
     // next use a word per (device, model), and the free capacity apart.
     using State = std::conditional_t<kReclaim != 0, uint32_t[kPer<Q>], DevState<Q>>;
     l.queue = o; o += round16((uint32_t)sizeof(State) * rs);
     l.free = o; o += kReclaim ? round16(4u * D * kP) : 0u;
-    l.open = o; o += round16(4u * kP);
-    l.flag = o; o += 16;
-    l.gmask = o; o += kReclaim ? 0u : round16(4u * Ring<kReclaim>::kBuffers * G::kG * kP);
+    l.open = o;
+    l.flag = o + 4u * kP; o += round16(4u * kP + 4u);
+    l.gmask = o; o += kReclaim ? 0u : round16(2u * Ring<kReclaim>::kBuffers * G::kG * kP);
     l.everl = o; o += kPhi && !kReclaim ? round16(2u * rs) : 0u;
     l.total = o;
     return l;
@@ -260,7 +258,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     int32_t *load = (int32_t *)(sm + L.load);
     uint32_t *arrival = (uint32_t *)(sm + L.arr);
     uint32_t *open = (uint32_t *)(sm + L.open);
-    uint32_t *gmask = (uint32_t *)(sm + L.gmask);  // [buffer][device group][plan]
+    uint16_t *gmask = (uint16_t *)(sm + L.gmask);  // [buffer][device group][plan]
     if (threadIdx.x < 16) weight[threadIdx.x] = (int)threadIdx.x < M ? __ldg(dp.weight + threadIdx.x) : 0;
     for (int32_t k = threadIdx.x; k < M * D; k += blockDim.x) load[k] = __ldg(dp.load + k);
     if (kReclaim) {
@@ -355,7 +353,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
 #pragma unroll
                 for (int gg = 0; gg < kG; ++gg) {
                     const uint32_t bal = __ballot_sync(0xFFFFFFFFu, key == (uint32_t)gg);
-                    if (pos == gg && qq[j] >= 0) gmask[(b * kG + gg) * kP + qq[j]] = (bal >> (kChunk * sub)) & 0xFFFFu;
+                    if (pos == gg && qq[j] >= 0) gmask[(b * kG + gg) * kP + qq[j]] = (uint16_t)(bal >> (kChunk * sub));
                 }
             }
 #pragma unroll
@@ -369,22 +367,23 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     } else if (warp >= 1) {
         // ---------------- residency (Eq. 11, Section 3.5) ----------------
         const int rl = (warp - 1) * 32 + lane;
-        constexpr int kRow = PcGroups<kP, kReclaim, Q>::kLanes;
+        constexpr int kRow = PcGroups<kP, kReclaim, Q>::kRow;
         if constexpr (!kReclaim) {
         // Lane (plan, device group): kG lanes per plan, and lane g plays the
         // plan's units on the devices d = g (mod kG) in dispatch order:
         // under least-recently-used reclamation devices do not interact.  The
         // producers leave each lane's units of the chunk as a mask (gmask).
-        const int qp = rl / kG, g = rl % kG;
-        const bool rmine = qp < kP;
+        // (plans side by side: the lanes' states lie in banks of their own)
+        const int qp = rl % kP, g = rl / kP;
+        const bool rmine = g < kG;
         const int64_t p = (rmine && qp < ng) ? (in_list ? (int64_t)in_list[j0 + qp] : j0 + qp) : 0;
         const bool live = rmine && qp < ng && out.status[p] == 0;
-        DevState<Q> *state = (DevState<Q> *)(sm + L.queue) + rl;  // [device / kG][lane]
-        uint16_t *everl = (uint16_t *)(sm + L.everl) + rl;        // [device / kG][lane], bit m: m was held (kPhi)
+        DevState<Q> *state = (DevState<Q> *)(sm + L.queue) + qp;  // [device][plan]
+        uint16_t *everl = (uint16_t *)(sm + L.everl) + qp;        // [device][plan], bit m: m was held (kPhi)
         if (rmine)
-            for (int32_t t = 0; t * kG + g < D; ++t) {
-                state[t * kRow].init((uint32_t)__ldg(dp.cap + t * kG + g));
-                if (kPhi) everl[t * kRow] = 0;
+            for (int32_t d = g; d < D; d += kG) {
+                state[d * kRow].init((uint32_t)__ldg(dp.cap + d));
+                if (kPhi) everl[d * kRow] = 0;
             }
         __syncthreads();
         for (int32_t c = 0; c < chunks; ++c) {
@@ -401,16 +400,16 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
                 const int32_t kn = todo ? __ffs((int)todo) - 1 : k;
                 const uint2 nv = rb[(1 * kChunk + kn) * kPitch];
                 const uint32_t r1 = v.x, r3 = v.y;
-                const int32_t t = (int32_t)(r3 & 31u) / kG;
-                DevState<Q> ds = state[t * kRow];
+                const int32_t d = (int32_t)(r3 & 31u);
+                DevState<Q> ds = state[d * kRow];
                 bool missed;
                 uint2 w = ds.settle(r1, r3, weight, load, D, dp.err, missed);
                 if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
-                    const uint32_t m = (r3 >> 5) & 15u, e = everl[t * kRow];
+                    const uint32_t m = (r3 >> 5) & 15u, e = everl[d * kRow];
                     w.x |= ((e >> m) & 1u) << 31;
-                    everl[t * kRow] = (uint16_t)(e | (1u << m));
+                    everl[d * kRow] = (uint16_t)(e | (1u << m));
                 }
-                state[t * kRow] = ds;
+                state[d * kRow] = ds;
                 rb[(1 * kChunk + k) * kPitch] = w;
                 k = kn;
                 v = nv;
@@ -419,7 +418,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         }
         if (live) {  // devices still occupied at the end
             uint32_t o = 0;
-            for (int32_t t = 0; t * kG + g < D; ++t) o += state[t * kRow].occupied();
+            for (int32_t d = g; d < D; d += kG) o += state[d * kRow].occupied();
             if (o) atomicAdd(open + qp, o);
         }
         } else {

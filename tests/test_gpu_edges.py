@@ -234,3 +234,25 @@ def test_placement_errors_found_by_the_sweep(reclaim):
     want = oracle_eval(prob, plans)
     assert (want["status"] & 2).any() and (want["status"] & 1).any() and (want["status"] == 0).any()
     assert_same(gpu_eval(prob, plans, k=8), want)
+
+
+@pytest.mark.parametrize("D,M", [(1, 9), (8, 12), (16, 16), (30, 9), (32, 12), (8, 4)])
+def test_last_window_of_the_64_bit_sweep(D, M):
+    """The largest window of one-activation sessions whose residency took a
+    weight, a queue and a count per device in CTAs of three plans (40-bit
+    finish slots) still starts in the 64-bit sweep when asked to."""
+    from test_gpu_reclaim import lone_sessions
+    wf = lib()
+    r16 = lambda x: (x + 15) & ~15
+    rs = 32 * -(-D // 10)
+
+    def size(W):
+        return (r16(4 * M) + r16(4 * D) + r16(4 * M * D) + r16(4 * W) + 4608 + r16(12 * (W + 2)) + r16(3 * (W + 2)) + r16(24 * D) +
+                r16(4 * rs) + r16((4 if M <= 8 else 8) * rs) + r16(rs) + 32 + 480)
+    W = next(w for w in range(14000, 1, -1) if size(w) <= 227 * 1024)
+    prob = lone_sessions(W, D, M, 20 * D + M)
+    plans = wfgen.make_plans(prob, 4, 1)
+    ctx = wf.Ctx(prob, max_P=4)
+    wf.wf_ctx_set_eval_path(ctx, wf.PATH_WIDE)
+    assert_same(gpu_eval(prob, plans, ctx=ctx), oracle_eval(prob, plans))
+    ctx.close()
