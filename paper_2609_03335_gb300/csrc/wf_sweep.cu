@@ -52,9 +52,14 @@ constexpr int kPlans32 = 16;                // plans per CTA of the u32 sweep
 // activations.  Named barriers: kFullP + b (producers -> residency), kFullR +
 // b (residency -> timing), kEmpty + b (timing -> producers) for buffer b;
 // kOpen (residency -> timing, once at the end).
+//
+// kReclaim, the reclamation order and who settles it: least recently used
+// (kLru), by next use with a lane per model (kNuModel), or by next use with a
+// lane per plan (kNuPlan, short windows in large batches).
+enum { kLru = 0, kNuModel = 1, kNuPlan = 2 };
 template <int kReclaim>
 struct Ring {
-    static constexpr int kBuffers = kReclaim ? 3 : 4;
+    static constexpr int kBuffers = kReclaim == kNuModel ? 3 : 4;
     static constexpr int kFullP = 1, kFullR = kFullP + kBuffers, kEmpty = kFullR + kBuffers, kOpen = kEmpty + kBuffers;
     static_assert(kOpen < 16, "named barriers");
 };
@@ -76,13 +81,13 @@ constexpr int kModelLanes = 2 * (int)sizeof(Q) / kPer<Q>;
 template <int kP, int kReclaim = 0, typename Q = uint32_t>
 struct PcShape {
     static constexpr int kProducers = kP >= 32 ? 8 : kP >= 16 ? 4 : kP >= 6 ? 3 : 2;
-    static constexpr int kRes = kReclaim ? (kP * kModelLanes<Q> + 31) / 32 : kP >= 32 ? 4 : kP >= 16 ? 2 : 1;  // residency warps
+    static constexpr int kRes = kReclaim == kNuModel ? (kP * kModelLanes<Q> + 31) / 32 : kReclaim == kNuPlan ? 2 : kP >= 32 ? 4 : kP >= 16 ? 2 : 1;  // residency warps
     static constexpr int kWarps = 1 + kRes + kProducers;
     // Four 16-plan CTAs share an SM (shared memory allows it at 2,000
     // activations), or four 6-plan CTAs at 8,192, which bounds the registers
     // per thread (large window with three of the latter, at 106 registers:
     // 56.0 ms, with four 47.4).
-    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP < 6 ? 1 : kP < 16 ? 4 : kReclaim && sizeof(Q) == 8 ? 3 : 4;
+    static constexpr int kMinBlocks = kP >= 32 ? 2 : kP < 6 ? 1 : kP < 16 ? 4 : kReclaim == kNuModel && sizeof(Q) == 8 ? 3 : kReclaim == kNuPlan ? 4 : 4;
     // Elements (8-byte word pairs) per (pair, position) row of the ring.  A
     // producer store covers 16 positions x 2 plans in two halves of 16
     // lanes; an odd pitch puts each half's 16 pairs on 32 distinct banks, and
@@ -99,7 +104,7 @@ template <int kP, int kReclaim, typename Q>
 struct PcGroups {
     using S = PcShape<kP, kReclaim, Q>;
     static constexpr int kG = kReclaim ? 1 : (32 * S::kRes) / kP;
-    static constexpr int kRow = kReclaim ? 32 * S::kRes : kP;  // row length of the state
+    static constexpr int kRow = kReclaim == kNuModel ? 32 * S::kRes : kP;  // row length of the state
     static_assert(kG >= 1 && kG * kP <= 32 * S::kRes, "residency lanes");
 };
 
@@ -149,7 +154,7 @@ struct PairArr {
 };
 
 struct PcLayout {
-    uint32_t weight, load, rcost, wsum, arr, ring, next, slots, slots_hi, tfree, free, queue, open, flag, gmask, everl, total;
+    uint32_t weight, load, rcost, wsum, arr, ring, next, slots, slots_hi, tfree, free, queue, open, flag, gmask, everl, nres, nuse, rcnt, total;
 };
 
 // Shared memory of a CTA of kP plans with TT times and NS slots per plan;
@@ -167,8 +172,8 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
     uint32_t o = 0;
     l.weight = o; o += 4u * 16;  // (zeros beyond M: read for the queue's empty places)
     l.load = o; o += round16(4u * M * D);
-    l.rcost = o; o += kReclaim ? round16(4u * M * D) : 0u;
-    l.wsum = o; o += kReclaim ? 256u * (uint32_t)sizeof(Q) : 0u;  // (the sums of each set of eight models; with Q of 16 bits more than the 16 used)
+    l.rcost = o; o += kReclaim == kNuModel ? round16(4u * M * D) : 0u;
+    l.wsum = o; o += kReclaim == kNuModel ? 256u * (uint32_t)sizeof(Q) : 0u;  // (the sums of each set of eight models; with Q of 16 bits more than the 16 used)
     l.arr = o; o += round16(4u * W);
     l.ring = o; o += round16(8u * Ring<kReclaim>::kBuffers * kPairs * kChunk * PcShape<kP>::kPitch);
     l.next = o; o += kReclaim ? round16(2u * Ring<kReclaim>::kBuffers * kChunk * PcShape<kP>::kPitch) : 0u;
@@ -178,13 +183,16 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
     const uint32_t rs = (uint32_t)(D * G::kRow);
     // Residency state: a word per device (DevState), or under reclamation by
     // next use a word per (device, model), and the free capacity apart.
-    using State = std::conditional_t<kReclaim != 0, uint32_t[kPer<Q>], DevState<Q>>;
+    using State = std::conditional_t<kReclaim == kNuModel, uint32_t[kPer<Q>], std::conditional_t<kReclaim == kNuPlan, Q, DevState<Q>>>;
     l.queue = o; o += round16((uint32_t)sizeof(State) * rs);
     l.free = o; o += kReclaim ? round16(4u * D * kP) : 0u;
     l.open = o;
     l.flag = o + 4u * kP; o += round16(4u * kP + 4u);
-    l.gmask = o; o += kReclaim ? 0u : round16(2u * Ring<kReclaim>::kBuffers * G::kG * kP);
-    l.everl = o; o += kPhi && !kReclaim ? round16(2u * rs) : 0u;
+    l.gmask = o; o += kReclaim == kNuModel ? 0u : round16(2u * Ring<kReclaim>::kBuffers * G::kG * kP);
+    l.everl = o; o += kPhi && kReclaim != kNuModel ? round16(2u * rs) : 0u;
+    l.nres = o; o += kReclaim == kNuPlan ? round16(rs) : 0u;
+    l.nuse = o; o += kReclaim == kNuPlan ? round16(2u * M * rs) : 0u;
+    l.rcnt = o; o += kReclaim == kNuPlan ? round16((uint32_t)M * kP) : 0u;
     l.total = o;
     return l;
 }
@@ -192,7 +200,7 @@ __host__ __device__ inline PcLayout pc_layout_q(int32_t D, int32_t M, int32_t W,
 template <int kP, typename TT, int kReclaim = 0, bool kPhi = false, typename ST = TT>
 inline PcLayout pc_layout(int32_t D, int32_t M, int32_t W, int32_t NS)
 {
-    if constexpr (kReclaim != 0)
+    if constexpr (kReclaim == kNuModel)
         if (M <= 4) return pc_layout_q<kP, TT, uint16_t, kReclaim, kPhi, ST>(D, M, W, NS);
     return M <= 8 ? pc_layout_q<kP, TT, uint32_t, kReclaim, kPhi, ST>(D, M, W, NS)
                   : pc_layout_q<kP, TT, uint64_t, kReclaim, kPhi, ST>(D, M, W, NS);
@@ -261,7 +269,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
     uint16_t *gmask = (uint16_t *)(sm + L.gmask);  // [buffer][device group][plan]
     if (threadIdx.x < 16) weight[threadIdx.x] = (int)threadIdx.x < M ? __ldg(dp.weight + threadIdx.x) : 0;
     for (int32_t k = threadIdx.x; k < M * D; k += blockDim.x) load[k] = __ldg(dp.load + k);
-    if (kReclaim) {
+    if (kReclaim == kNuModel) {
         for (uint32_t k = threadIdx.x; k < 64u * sizeof(Q); k += blockDim.x) {
             uint32_t w = 0;
             for (int32_t m = 0; m < 8; ++m)
@@ -348,7 +356,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
             // For each residency lane, the chunk's units on its devices: one
             // ballot per device group; each half-warp holds one plan.
 #pragma unroll
-            for (int j = 0; j < kIters && !kReclaim; ++j) {
+            for (int j = 0; j < kIters && kReclaim != kNuModel; ++j) {
                 const uint32_t key = dev[j] == 0xFFFFFFFFu ? (uint32_t)kG : dev[j] % kG;
 #pragma unroll
                 for (int gg = 0; gg < kG; ++gg) {
@@ -368,7 +376,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         // ---------------- residency (Eq. 11, Section 3.5) ----------------
         const int rl = (warp - 1) * 32 + lane;
         constexpr int kRow = PcGroups<kP, kReclaim, Q>::kRow;
-        if constexpr (!kReclaim) {
+        if constexpr (kReclaim == kLru) {
         // Lane (plan, device group): kG lanes per plan, and lane g plays the
         // plan's units on the devices d = g (mod kG) in dispatch order:
         // under least-recently-used reclamation devices do not interact.  The
@@ -419,6 +427,101 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         if (live) {  // devices still occupied at the end
             uint32_t o = 0;
             for (int32_t d = g; d < D; d += kG) o += state[d * kRow].occupied();
+            if (o) atomicAdd(open + qp, o);
+        }
+        } else if constexpr (kReclaim == kNuPlan) {
+        // By next use with a lane per plan: the same rules as below, a victim at
+        // a time, each found by a scan of the device's queue.  A longer chain
+        // for one plan, but fewer instructions in all (lane_per_plan says where).
+        constexpr int kEvery = 32 * S::kRes / kP;  // the lanes that play, spread over the residency warps
+        const int qp = rl / kEvery;
+        const bool rmine = rl % kEvery == 0;
+        const int64_t p = (rmine && qp < ng) ? (in_list ? (int64_t)in_list[j0 + qp] : j0 + qp) : 0;
+        const bool live = rmine && qp < ng && out.status[p] == 0;
+        Q *queue = (Q *)(sm + L.queue) + qp;               // [device][plan]: resident models, least recently used first
+        uint8_t *nres = sm + L.nres + qp;                  // [device][plan]: how many
+        uint32_t *room = (uint32_t *)(sm + L.free) + qp;   // [device][plan]: free capacity
+        uint16_t *nuse = (uint16_t *)(sm + L.nuse) + qp;   // [device][model][plan]: next use of the copy there
+        uint8_t *copies = sm + L.rcnt + qp;                // [model][plan]: devices that hold it
+        uint16_t *everl = (uint16_t *)(sm + L.everl) + qp; // [device][plan], bit m: m was held (kPhi)
+        if (rmine) {
+            for (int32_t d = 0; d < D; ++d) {
+                queue[d * kP] = 0;
+                nres[d * kP] = 0;
+                room[d * kP] = (uint32_t)__ldg(dp.cap + d);
+                if (kPhi) everl[d * kP] = 0;
+            }
+            for (int32_t m = 0; m < M; ++m) copies[m * kP] = 0;
+        }
+        __syncthreads();
+        for (int32_t c = 0; c < chunks; ++c) {
+            const int b = c % kBuffers;
+            named_sync(kFullP + b, kProdThreads + kResThreads);
+            uint2 *rb = ring + b * kRW * kChunk * kPitch + (rmine ? qp : 0);
+            const uint16_t *nb = next + b * kChunk * kPitch + (rmine ? qp : 0);
+            for (uint32_t todo = live ? gmask[b * kP + qp] : 0u; todo; todo &= todo - 1) {
+                const int32_t k = __ffs((int)todo) - 1, here = c * kChunk + k;
+                const uint2 v = rb[(1 * kChunk + k) * kPitch];
+                const uint32_t r1 = v.x, r3 = v.y, m = (r3 >> 5) & 15u, wm = (uint32_t)weight[m];
+                const int32_t d = (int32_t)(r3 & 31u);
+                Q q = queue[d * kP];
+                uint32_t n = nres[d * kP], f = room[d * kP];
+                const bool was_empty = n == 0;
+                const int32_t at = Lru<Q>::find(q, n, m);
+                const bool hit = at < (int32_t)n;
+                q = hit ? Lru<Q>::remove(q, hit ? at : 0) : q;
+                n -= hit ? 1u : 0u;
+                const uint32_t need = hit ? r1 : wm + r1;  // at most the capacity
+                while (need > f && n > 0) {
+                    // A copy also held elsewhere goes first, then an infinite
+                    // quotient, then the larger one (exact products), then the
+                    // earlier entry.
+                    int32_t best = 0, bdist = 0, bcost = 0;
+                    uint32_t bclass = 0;
+#pragma unroll
+                    for (int32_t e = 0; e < Lru<Q>::kSlots; ++e) {
+                        if (e >= (int32_t)n) break;
+                        const uint32_t x = (uint32_t)(q >> (4 * e)) & 15u;
+                        const int32_t nu = nuse[(d * M + x) * kP], cost = load[x * D + d], dist = nu - here;
+                        const bool inf = nu == 0xFFFF || cost == 0;
+                        const uint32_t cls = (copies[x * kP] > 1 ? 2u : 0u) | (inf ? 1u : 0u);
+                        if (e == 0 || cls > bclass || (cls == bclass && !inf && (int64_t)dist * bcost > (int64_t)bdist * cost)) {
+                            best = e; bclass = cls; bdist = dist; bcost = cost;
+                        }
+                    }
+                    const uint32_t x = (uint32_t)(q >> (4 * best)) & 15u;
+                    f += (uint32_t)weight[x];
+                    copies[x * kP] -= 1;
+                    q = Lru<Q>::remove(q, best);
+                    n -= 1;
+                }
+                if (need > f) atomicExch(dp.err, 2);  // unreachable for a valid plan
+                uint2 w = settled(r3, hit, (uint32_t)load[m * D + d], was_empty, (r3 & kDrop) != 0 && n == 0);
+                if (kPhi && !hit) {
+                    const uint32_t e = everl[d * kP];
+                    w.x |= ((e >> m) & 1u) << 31;
+                    everl[d * kP] = (uint16_t)(e | (1u << m));
+                }
+                if (r3 & kDrop) {  // the model leaves when the unit ends
+                    f += hit ? wm : 0u;
+                    copies[m * kP] -= hit ? 1 : 0;
+                } else {
+                    f -= hit ? 0u : wm;
+                    copies[m * kP] += hit ? 0 : 1;
+                    nuse[(d * M + m) * kP] = nb[k * kPitch];
+                    q |= (Q)m << (4 * n);
+                    n += 1;
+                }
+                queue[d * kP] = q;
+                nres[d * kP] = (uint8_t)n;
+                room[d * kP] = f;
+                rb[(1 * kChunk + k) * kPitch] = w;
+            }
+            named_arrive(kFullR + b, kResThreads + 32);
+        }
+        if (live) {  // devices still occupied at the end
+            uint32_t o = 0;
+            for (int32_t d = 0; d < D; ++d) o += nres[d * kP] != 0;
             if (o) atomicAdd(open + qp, o);
         }
         } else {
@@ -1159,7 +1262,7 @@ template <typename TT, int kR, typename F>
 int pc_visit(const wf_dev_problem &dp, int kp, F &&f)
 {
     auto by_q = [&](auto p, auto s) {
-        if constexpr (kR != 0)
+        if constexpr (kR == kNuModel)
             if (dp.M <= 4) return f(Ty<uint16_t>{}, p, s);
         return dp.M <= 8 ? f(Ty<uint32_t>{}, p, s) : f(Ty<uint64_t>{}, p, s);
     };
@@ -1284,6 +1387,23 @@ int launch_pc_q(const wf_ctx *ctx, int kp, int resident, const wf_plans *pl, con
 }
 
 }  // namespace
+
+// Whether reclamation by next use settles with a lane per plan: short windows in
+// batches large enough that the instructions of all plans bound the sweep and
+// not the chain of one.  A model's lanes cost the same whether a unit evicts or
+// not, a plan's lane the more the fewer devices share the models: the more
+// devices, the longer the windows that it wins.  us with a lane per model and
+// with a lane per plan, 30,000 and 90,000 plans: D = 8, M = 8, N = 24 123 and 122, 273 and
+// 261; N = 64 214 and 235, 521 and 551.  D = 14, M = 5, N = 40 149 and 148, 348 and 330;
+// N = 64 196 and 203, 476 and 474.  D = 8, M = 12, N = 64 294 and 290, 750 and 698; N = 128
+// 575 and 611, 1,549 and 1,516.  D = 16, M = 12, N = 128 571 and 574, 1,534 and 1,418.  4,000
+// plans of D = 8, M = 12, N = 64: 82 and 93; 8,000: 121 and 103.  Up to four models four
+// lanes a plan win from N = 24 on, and lose 2 % below.
+static bool lane_per_plan(const wf_ctx *ctx, int64_t P)
+{
+    const wf_dev_problem &dp = ctx->dp;
+    return dp.reclaim && dp.M > 4 && P > 40 * (int64_t)ctx->sms && dp.N <= (dp.M <= 8 ? 24 + 2 * dp.D : 32 + 8 * dp.D);
+}
 
 int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st)
 {
@@ -1436,7 +1556,16 @@ int wf_launch_sweep(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, con
     } else if (cfg.smem32 && !(wide_first && cfg.smem64)) {
         // u32 times for every plan; the plans that leave 32 bits go on to the
         // u64 sweep, and from there (or straight) to the int64 path.
-        rc = launch_pc_q<uint32_t>(ctx, kPlans32, cfg.res32, pl, out, cfg.smem32, nullptr, nullptr, list1, counts, st);
+        const wf_dev_problem &dp = ctx->dp;
+        const bool by_plan = lane_per_plan(ctx, pl->P);
+        const size_t smem = !by_plan      ? cfg.smem32
+                            : dp.phi_life ? pc_layout<kPlans32, uint32_t, kNuPlan, true>(dp.D, dp.M, dp.W, dp.nslots + 2).total
+                                          : pc_layout<kPlans32, uint32_t, kNuPlan, false>(dp.D, dp.M, dp.W, dp.nslots + 2).total;
+        if (by_plan)
+            rc = dp.phi_life ? launch_pc_r<uint32_t, kNuPlan, true>(ctx, kPlans32, 1, pl, out, smem, nullptr, nullptr, list1, counts, st)
+                             : launch_pc_r<uint32_t, kNuPlan, false>(ctx, kPlans32, 1, pl, out, smem, nullptr, nullptr, list1, counts, st);
+        else
+            rc = launch_pc_q<uint32_t>(ctx, kPlans32, cfg.res32, pl, out, smem, nullptr, nullptr, list1, counts, st);
         if (rc) return rc;
         if (!cfg.smem64) { *rest_list = list1; *rest_count = counts; return WF_OK; }
         rc = launch_pc_q<uint64_t>(ctx, cfg.plans64, cfg.res64, pl, out, cfg.smem64, list1, counts, list2, counts + 1, st);

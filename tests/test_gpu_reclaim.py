@@ -125,6 +125,36 @@ def test_window_lengths_of_the_next_use_pass(n):
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
 
 
+@pytest.mark.parametrize("D,M,scale,shift", [(2, 5, 1, 0), (8, 8, 1, 0), (9, 9, 1, 0), (32, 16, 1, 0), (4, 6, 400000, 3_000_000_000),
+                                             (3, 12, 1 << 20, 1_500_000_000)])
+def test_short_windows_in_large_batches(D, M, scale, shift):
+    """Batches of more than 40 plans an SM, where windows up to a length take a
+    lane per plan: the longest such window and the next longer one, the batch at
+    the limit and one plan more; all rules of the order, window terms, retain
+    rows, invalid plans, run times that leave 32 bits."""
+    import torch
+    from test_gpu_phi import check
+    most = 40 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(3500 + 10 * D + M)
+    limit = 24 + 2 * D if M <= 8 else 32 + 8 * D
+    for n in (limit, limit + 1, 9):
+        cuts = [n] if n < 20 else [n // 3, n // 3, n - 2 * (n // 3)]
+        sess = [(wfgen.fam_softdev(c), wfgen.fam_research(c, width=3), wfgen.fam_layered(c, rng, width=3))[i % 3] for i, c in enumerate(cuts)]
+        dev = wfgen.DeviceSpec(cap_gib=[(60 + 7 * d) / wfgen.GIB for d in range(D)], speed=[1.0 + 0.1 * d for d in range(D)], bw_gbps=[1] * D)
+        prob = wfgen.assemble("short", sess, shift + np.sort(rng.integers(0, 300, len(sess))).astype(np.int64), dev,
+                              [(5 + (7 * m) % 31) / wfgen.GIB for m in range(M)], rng, lat_median_us=100, lat_sigma=0.6, kv_lo=1, kv_hi=20)
+        assert prob.N == n
+        prob = prob.with_(load_us=rng.integers(0, 60, M * D).astype(np.int32), reclaim=1,
+                          lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, 1 << 26).astype(np.int32))
+        plans = wfgen.make_plans(prob, most + 1, D + M, p_retain=0.8 if D % 2 else None)
+        plans.place[7, 0] = D
+        plans.order[11, 0] = plans.order[11, 1]
+        got = check(prob, plans, k=8, reclaim=1)
+        plain = gpu_eval(prob, plans)
+        assert_same(plain, got)
+        assert_same(gpu_eval(prob, plans.slice(0, most)), {x: got[x][:most] for x in ("status", "makespan", "p95", "gpu")})
+
+
 def lone_sessions(W, D, M, seed):
     """W sessions of one activation each: as many finish slots as sessions."""
     rng = np.random.default_rng(seed)
