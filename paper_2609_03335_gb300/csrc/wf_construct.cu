@@ -43,14 +43,14 @@ constexpr int kWarpsPerSm = kWarps * kCtasPerSm;
 // Lanes per plan.  The chain of one plan is shorter on more lanes (a warp's
 // minimum is two reductions, a longer ready set takes fewer rounds), the
 // chip's issue slots hold more plans on fewer.  N = 1,000, D = 3, us with 8,
-// 16, 32 lanes: 512 plans 1,267, 1,128, 928; 1,024: 1,278, 1,130, 988; 2,048: 1,291,
-// 1,234, 1,311; 3,072: 1,535, 1,450, 1,804; 4,096: 1,588, 1,676, 2,075.  N = 40 to
-// 2,000 with 3 and 8 devices change sides at the same batches, 8 and 24 plans an
+// 16, 32 lanes: 512 plans 1,267, 1,128, 928; 1,024: 1,278, 1,130, 988; 1,766: 16
+// lanes 1,220, 32 lanes 1,113; 2,048: 1,291, 1,234, 1,311; 3,072: 1,535, 1,450, 1,804; 4,096: 1,588, 1,676, 2,075.  N = 40 to
+// 2,000 with 3 and 8 devices change sides at the same batches, 12 and 24 plans an
 // SM.
 int lanes_of(int32_t D, int64_t P, int sms)
 {
     const int least = D <= 8 ? 8 : D <= 16 ? 16 : 32;
-    return std::max(least, P <= 8 * (int64_t)sms ? 32 : P <= 24 * (int64_t)sms ? 16 : 8);
+    return std::max(least, P <= 12 * (int64_t)sms ? 32 : P <= 24 * (int64_t)sms ? 16 : 8);
 }
 
 __device__ __forceinline__ uint64_t mix64(uint64_t x)  // SplitMix64 output function

@@ -93,7 +93,7 @@ def test_the_last_ready_entry_is_taken(lengths, D, P):
 
 @pytest.mark.parametrize("D,M", [(5, 8), (8, 9), (13, 4), (16, 9)])
 def test_lanes_by_batch(D, M):
-    """The batches at which a plan takes 32, 16 or 8 lanes (8 and 24 plans an
+    """The batches at which a plan takes 32, 16 or 8 lanes (12 and 24 plans an
     SM), and one more plan each, on one context made for the largest; the same
     seed gives the same plans whatever the lanes."""
     import torch
@@ -104,7 +104,7 @@ def test_lanes_by_batch(D, M):
     most = 24 * sms + 1
     ctx = wf.Ctx(prob, max_P=most)
     want, _ = oracle.construct(prob, most, seed=6, jitter=700)
-    for P in (most, 24 * sms, 8 * sms + 1, 8 * sms, 3):
+    for P in (most, 24 * sms, 12 * sms + 1, 12 * sms, 3):
         out = wf.DevicePlans.empty(P, prob.N)
         wf.wf_construct_plans(ctx, out, 6, 700)
         torch.cuda.synchronize()
