@@ -120,6 +120,27 @@ def test_times_past_32_bits(scale, B):
     ctx.close()
 
 
+@pytest.mark.parametrize("D,B", [(3, 4), (12, 6), (24, 2)])
+def test_many_plans_past_32_bits(D, B):
+    """More plans leave 32 bits than the CTAs of the 64-bit sweep hold at once
+    (six an SM of eight plans each), so each walks over several groups; a
+    third of the plans stay within 32 bits, and some are invalid."""
+    import torch
+    P = 60 * torch.cuda.get_device_properties(0).multi_processor_count * 3 // 2
+    rng = np.random.default_rng(3700 + D)
+    prob = random_problem(rng, n_sessions=2, sizes=(5, 6), D=D, M=5).with_(batch=B)
+    base = oracle_eval(prob, wfgen.make_plans(prob, 300, 6))
+    ok = base["status"] == 0
+    shift = (1 << 32) - int(np.quantile(base["makespan"][ok], 0.3)) - int(prob.arrival_us.min())  # (a third of the plans end below 2^32)
+    prob = prob.with_(arrival_us=prob.arrival_us + shift)
+    plans = wfgen.make_plans(prob, P, 6)
+    inject_invalid(plans, prob, rng, frac=0.02)
+    want = oracle_eval(prob, plans)
+    end = want["makespan"][want["status"] == 0] + int(prob.arrival_us.min())
+    assert 0.1 < (end < (1 << 32)).mean() < 0.6
+    assert_same(_gpu(prob, plans), want)
+
+
 def test_refusals():
     wf = lib()
     import torch

@@ -38,3 +38,17 @@ def test_sample_counts_shapes_and_tables(S, P, D, M, kind):
     if P >= 8:
         inject_invalid(plans, prob, rng)
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
+
+
+@pytest.mark.parametrize("S,P,D,M", [(20, 3000, 3, 4), (33, 2600, 9, 9), (64, 2500, 4, 5), (65, 2000, 5, 8), (129, 1500, 3, 10), (256, 1400, 2, 4)])
+def test_teams_that_play_several_plans(S, P, D, M):
+    """Short windows and enough plans that every team plays several in the same
+    shared memory (at least one more than the chip holds at once), one and two
+    samples a lane, one to four timing warps, invalid plans between the others."""
+    rng = np.random.default_rng(9500 + S)
+    prob = random_problem(rng, n_sessions=2, sizes=(5, 7), D=D, M=M)
+    r, c, e = tables("short")
+    prob = prob.with_(S=S, seed=int(rng.integers(0, 2**63)), bm_r=r, bm_c=c, bm_e=e)
+    plans = wfgen.make_plans(prob, P, S, p_retain=0.6 if S % 2 else None)
+    inject_invalid(plans, prob, rng)
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
