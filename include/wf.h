@@ -68,7 +68,8 @@ enum {
 /* Evaluation path (wf_ctx_set_eval_path). */
 enum {
     WF_PATH_AUTO = 0,     /* the shared-memory sweeps, the exact int64 path for what they hand on (the default) */
-    WF_PATH_INT64 = 1,    /* every plan on the exact int64 path (a thread per plan, state in global memory) */
+    WF_PATH_INT64 = 1,    /* every plan on the exact int64 path (a warp per plan; under a replica batch limit a
+                             thread per plan, of a stochastic window a thread per sample) */
     WF_PATH_WIDE = 2,     /* every plan starts in the 64-bit sweep */
     WF_PATH_RELATIVE = 3  /* every plan starts in the sweep with 32-bit times relative to a per-plan base */
 };
@@ -374,8 +375,8 @@ int wf_local_search(wf_ctx *ctx, const wf_plans *elite, const wf_eval_out *elite
  * Retain rows, if given, are set to all ones.  WF_EINVAL when the window's
  * horizon (latest arrival + every node's worst load + run + grant) plus
  * jitter_us reaches 2^47 us.  The first call on a context allocates the
- * constructor's state (about 20 N bytes per plan built at once, at most
- * 128 plans per SM); later calls allocate nothing.  Asynchronous on stream.
+ * constructor's state (18 N bytes per plan built at once, at most 112 plans
+ * per SM); later calls allocate nothing.  Asynchronous on stream.
  */
 int wf_construct_plans(wf_ctx *ctx, const wf_plans *out, uint64_t seed, int64_t jitter_us, void *stream);
 

@@ -28,7 +28,7 @@
 // weights).  Control flow is uniform over the warp: a loop runs until every
 // plan of the warp is through.  Bound by integer issue (64-bit hashes, keys
 // and times).  16,384 plans of the burst window (N = 2,000, D = 8, jitter
-// 0.2 s): 17.9 ms with a warp per plan (13.7 G warp instructions), 6.46 ms with 8
+// 0.2 s): 17.9 ms with a warp per plan (13.7 G warp instructions), 6.34 ms with 8
 // lanes per plan (4.8 G, 63 % of the issue slots).
 #include <algorithm>
 

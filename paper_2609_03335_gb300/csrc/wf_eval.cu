@@ -1,4 +1,4 @@
-// Plan evaluation (rows a3-a11): status bits, then a list-schedule play of
+// Plan evaluation: status bits, then a list-schedule play of
 // each plan over the window with fused chains (Eq. 3-4), releases (Eq. 2,
 // Eq. 7), per-device order (Eq. 10), LRU residency under capacity (Eq. 11),
 // loads / prefetches on the consumer's device (Eq. 5, Eq. 9), retain /
@@ -400,9 +400,10 @@ __device__ __forceinline__ int32_t p95_rank(int64_t n) { return (int32_t)((95 * 
 // other plans' warps.  Times are TT: u64 on the int64 path; the static entry
 // point plays u32 first, with half the memory and a third of the instructions
 // per maximum, and again on u64 only the plans that leave 32 bits.  1,900
-// plans of N = 2,000 in wf_eval_plans_static: 14.3 ms with a thread per plan
+// plans of N = 2,000 in wf_eval_plans_static: 14.2 ms with a thread per plan
 // and its state in global memory, 0.81 ms with a warp per plan on 64-bit
-// times (108 warp instructions per plan-position), 0.57 ms on u32 times (80).
+// times, 0.57 ms on u32 times, 0.53 ms with the devices' state in one word
+// each (73 warp instructions per plan-position; 93 on 64-bit times).
 // ---------------------------------------------------------------------------
 
 // The warp's working memory: B's answers for C [32], the models' weights [16],

@@ -1,4 +1,4 @@
-// Stochastic latencies (row a11): the plans of a window with S latency
+// Stochastic latencies: the plans of a window with S latency
 // samples, each sample's times on u32; the floor means over the samples and the
 // nearest-rank p95 of all their sessions' latencies.
 //

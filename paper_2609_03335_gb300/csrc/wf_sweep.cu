@@ -1,4 +1,4 @@
-// Plan evaluation in shared memory (rows a3-a11).
+// Plan evaluation in shared memory.
 //
 // Deterministic plans (pc_kernel): a CTA plays 16 plans as a three-stage warp
 // pipeline over 16 dispatch positions at a time.  Producer warps turn each
@@ -537,9 +537,12 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
         // once, by a float quotient, and a copy goes if those before it do
         // not make room enough; where the float cannot tell two quotients
         // apart (its error is below 2^-21) exact products decide.  The stage
-        // is bound by issue (about 200 instructions a unit of four plans).
+        // is bound by issue (about 200 instructions a unit of four plans).  Nine
+        // warps in four CTAs leave 56 registers a thread up to eight models, of
+        // which the producers' and this loop spill 120 bytes; three producer warps
+        // (64 registers) spill 240 and take 2,706, two 3,345, three CTAs 2,992.
         // 16,384 plans of N = 2,000, D = M = 8, us a step: a lane per plan, which
-        // scanned the queue for each victim, 4,095; a lane per model 2,722; two
+        // scanned the queue for each victim, 4,095; a lane per model 2,629; two
         // models a lane (270 instructions for eight plans, half the warps) 3,010;
         // a lane per model with a loop that takes one victim at a time 3,172.
         // Up to four models half the lanes would idle: four lanes a plan, two
@@ -960,7 +963,7 @@ pc_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, const int32_t *in_lis
 // chunks of gathers are in flight ahead of the one being settled; one or two
 // chunks have nothing to run ahead of, and what bounds those is the plans an
 // SM holds: 32 registers instead of 48, no read for a position that is not
-// there.  39,692 plans of N = 22, us: 18.3 with the deep form, 12.0 without; the
+// there.  39,692 plans of N = 22, us: 18.3 with the deep form, 12.5 without; the
 // call on 30,000 plans of N = 32, D = M = 8 137 and 134, of N = 64 212 and 209, and
 // from N = 128 on the deep form is ahead (355 and 359).
 constexpr int kNuWarps = 4;

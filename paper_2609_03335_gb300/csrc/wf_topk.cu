@@ -1,4 +1,4 @@
-// Top-k of evaluated plans (row a12) by the key (status != 0, makespan, p95,
+// Top-k of evaluated plans by the key (status != 0, makespan, p95,
 // gpu, plan index), ascending.
 //
 //  1. threshold: T, a 64-bit key (status != 0) << 63 | makespan that at
