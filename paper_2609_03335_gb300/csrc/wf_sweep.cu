@@ -1400,12 +1400,17 @@ int launch_pc_q(const wf_ctx *ctx, int kp, int resident, const wf_plans *pl, con
 // 261; N = 64 214 and 235, 521 and 551.  D = 14, M = 5, N = 40 149 and 148, 348 and 330;
 // N = 64 196 and 203, 476 and 474.  D = 8, M = 12, N = 64 294 and 290, 750 and 698; N = 128
 // 575 and 611, 1,549 and 1,516.  D = 16, M = 12, N = 128 571 and 574, 1,534 and 1,418.  4,000
-// plans of D = 8, M = 12, N = 64: 82 and 93; 8,000: 121 and 103.  Up to four models four
+// plans of D = 8, M = 12, N = 64: 82 and 93; 8,000: 121 and 103.  (All with about 20
+// activations a session.)  Long sessions, whose chains keep to few models, evict
+// less too: D = 3, M = 6, N = 64 in one session 166 and 164, 397 and 376, N = 80 in two
+// 198 and 198, 487 and 465, but N = 64 in three 209 and 244, 505 and 571; M = 5,
+// D = 3, N = 80 in two 480 and 462.  Up to four models four
 // lanes a plan win from N = 24 on, and lose 2 % below.
 static bool lane_per_plan(const wf_ctx *ctx, int64_t P)
 {
     const wf_dev_problem &dp = ctx->dp;
-    return dp.reclaim && dp.M > 4 && P > 40 * (int64_t)ctx->sms && dp.N <= (dp.M <= 8 ? 24 + 2 * dp.D : 32 + 8 * dp.D);
+    if (!dp.reclaim || dp.M <= 4 || P <= 40 * (int64_t)ctx->sms) return false;
+    return dp.N <= (dp.M > 8 ? 32 + 8 * dp.D : dp.N >= 32 * dp.W ? 96 : 24 + 2 * dp.D);
 }
 
 int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st)

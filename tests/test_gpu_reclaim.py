@@ -155,6 +155,22 @@ def test_short_windows_in_large_batches(D, M, scale, shift):
         assert_same(gpu_eval(prob, plans.slice(0, most)), {x: got[x][:most] for x in ("status", "makespan", "p95", "gpu")})
 
 
+@pytest.mark.parametrize("n,sessions", [(96, 3), (97, 3), (96, 1), (95, 3), (64, 2)])
+def test_long_sessions_in_large_batches(n, sessions):
+    """Up to eight models, windows of up to 96 activations take a lane per plan
+    when their sessions have 32 or more: at and around both limits."""
+    import torch
+    P = 40 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    rng = np.random.default_rng(3600 + n + sessions)
+    prob = random_problem(rng, n_sessions=sessions, sizes=(n // sessions,) * 2, D=3, M=6)
+    while prob.N != n:  # (the families round some sizes)
+        prob = random_problem(rng, n_sessions=sessions, sizes=(n // sessions, n // sessions + (n % sessions > 0)), D=3, M=6)
+    prob = prob.with_(reclaim=1)
+    plans = wfgen.make_plans(prob, P, n)
+    plans.place[7, 0] = 3
+    assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
+
+
 def lone_sessions(W, D, M, seed):
     """W sessions of one activation each: as many finish slots as sessions."""
     rng = np.random.default_rng(seed)
