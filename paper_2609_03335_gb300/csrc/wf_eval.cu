@@ -7,7 +7,8 @@
 // Mapping: a warp plays a deterministic plan (warp_play); for
 // wf_eval_plans_phi it also returns the window terms of Eq. 12's ranking key
 // (timely prefetches, lifecycle overhead).  One thread plays one (plan, sample)
-// of a stochastic window, or one plan under the replica batch limit: its
+// of a stochastic window, one plan under the replica batch limit, or one plan
+// of a large batch of short windows on few devices: its
 // mutable state (chain-tail finish times, per-device and per-session state)
 // lives in a scratch row of the context, and plans beyond the number of rows
 // are taken in rounds.
@@ -124,12 +125,14 @@ __device__ __forceinline__ uint64_t splitmix(uint64_t x)
     return x ^ (x >> 31);
 }
 
-// Run time of activation n on device d in a latency sample: scaled by the
-// multiplier drawn from (plan, sample, n) through the integer Box-Muller
+// Run time of activation n on device d; in a latency sample (kStoch) scaled by
+// the multiplier drawn from (plan, sample, n) through the integer Box-Muller
 // tables (an arithmetic right shift of the signed product is the floor).
+template <bool kStoch>
 __device__ __forceinline__ int64_t run_time(const wf_dev_problem &dp, int32_t n, int32_t d, uint64_t key)
 {
     const int64_t base = dp.lat[(int64_t)n * dp.D + d];
+    if (!kStoch) return base;
     const uint64_t h = splitmix(key ^ (uint64_t)n);
     const int64_t r = dp.bm_r[h & (uint64_t)(dp.bm_rn - 1)];
     const int64_t c = dp.bm_c[(h >> 32) & (uint64_t)(dp.bm_cn - 1)];
@@ -138,9 +141,10 @@ __device__ __forceinline__ int64_t run_time(const wf_dev_problem &dp, int32_t n,
     return (base * mult + 32768) >> 16;
 }
 
-// One play of a valid plan for one latency sample by one thread.  Returns
-// makespan and GPU time; per-session completion latencies are left in
-// row.comp.
+// One play of a valid plan (kStoch: for one latency sample) by one thread.
+// Returns makespan, counted from dp.first_arrival, and GPU time; per-session
+// completion latencies are left in row.comp.
+template <bool kStoch>
 __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uint64_t key,
                      int64_t *makespan, int64_t *gpu_total)
 {
@@ -170,10 +174,10 @@ __device__ void play(const wf_dev_problem &dp, const PlanRows &pr, Row &row, uin
         const int32_t wm = dp.weight[m];
         int32_t tail = h;
         int64_t kv = dp.peak[(int64_t)h * D + d] - wm;
-        int64_t run = run_time(dp, h, d, key);
+        int64_t run = run_time<kStoch>(dp, h, d, key);
         for (int32_t s = dp.fnext[h]; s >= 0 && bit_at(pr.fuse, s) && pr.place[s] == d; s = dp.fnext[s]) {
             kv = max(kv, (int64_t)dp.peak[(int64_t)s * D + d] - wm);
-            run += run_time(dp, s, d, key);
+            run += run_time<kStoch>(dp, s, d, key);
             tail = s;
         }
 
@@ -567,7 +571,7 @@ __device__ bool warp_play(const wf_dev_problem &dp, const PlanRows &pr, const Wa
             const uint32_t r1 = __shfl_sync(0xFFFFFFFFu, (uint32_t)kv, k), r3 = __shfl_sync(0xFFFFFFFFu, w3, k);
             if (mine) {
                 bool missed;
-                uint2 x = ds.settle(r1, r3, wm.weight, dp.load, D, dp.err, missed);
+                uint2 x = ds.template settle<true>(r1, r3, wm.weight, dp.load, D, dp.err, missed);
                 if (kPhi && missed) {  // a reload of a model this device held before: bit 31 of the load word
                     const uint32_t mk = (r3 >> 5) & 15u;
                     x.x |= ((ever >> mk) & 1u) << 31;
@@ -683,6 +687,20 @@ WarpShape warp_shape(int sms, int64_t P, size_t bytes, int solo)
     return fit < solo && P > fit * sms ? kRows : kSolo;
 }
 
+// Whether large batches of short windows on few devices play with a thread per
+// plan instead: a warp settles the devices' units side by side, and with up to
+// four devices it mostly waits for one of them, while N and D that small keep
+// a thread's row in L1 and L2.  60,000 plans in wf_eval_plans_static, us, a
+// warp and a thread per plan: D = 2, N = 14 144 and 94, N = 39 270 and 175, N = 64
+// 332 and 323, N = 100 367 and 427; D = 3, N = 39 223 and 186, N = 64 230 and 277; D = 4,
+// N = 24 146 and 130, N = 39 184 and 214; D = 5, N = 14 102 and 106.  22,076 plans of D = 2,
+// N = 39 about the same either way: a thread's chain is longer.  On 64-bit times
+// (wide) a warp gains less: 60,000 plans of D = 4, N = 39 297 and 242.
+bool thread_per_plan(const wf_dev_problem &dp, int sms, int64_t P, bool wide)
+{
+    return dp.D <= 4 && (int64_t)dp.N * dp.D <= (wide ? 160 : 120) && P > 160 * (int64_t)sms;
+}
+
 // Every plan of the batch, or (list) the plans whose times a sweep could not
 // hold, on int64 times; a warp walks over plans.
 template <typename Q, bool kPhi, WarpShape kShape>
@@ -706,10 +724,11 @@ eval_warp_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scrat
     }
 }
 
-// The replica batch limit on the int64 path: a thread per plan, rows of
-// global scratch; every plan, or the listed ones.
+// A thread per plan on the int64 path, rows of global scratch; every plan, or
+// the listed ones: the replica batch limit (kBatched), or thread_per_plan().
+template <bool kBatched>
 __global__ void __launch_bounds__(kEvalThreads)
-eval_batched_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
+eval_thread_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scratch, size_t row_bytes,
                     int64_t rows, const int32_t *list, const int32_t *count)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -726,7 +745,8 @@ eval_batched_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *sc
             continue;
         }
         int64_t mk, g;
-        play_batched(dp, pr, row, &mk, &g);
+        if (kBatched) play_batched(dp, pr, row, &mk, &g);
+        else play<false>(dp, pr, row, 0, &mk, &g);
         out.makespan_us[p] = mk;
         out.gpu_us[p] = g;
         out.p95_us[p] = select_rank(row.comp, dp.W, p95_rank(dp.W));
@@ -772,7 +792,7 @@ eval_stoch_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *scra
         for (int32_t s = threadIdx.x; s < S; s += blockDim.x) {
             const uint64_t key = splitmix(splitmix(dp.seed ^ gp) ^ (uint64_t)s);
             int64_t mk, g;
-            play(dp, pr, row, key, &mk, &g);
+            play<true>(dp, pr, row, key, &mk, &g);
             atomicAdd(&s_mk, (unsigned long long)mk);
             atomicAdd(&s_gpu, (unsigned long long)g);
             for (int32_t w = 0; w < W; ++w) pool[(int64_t)s * W + w] = row.comp[w];
@@ -846,10 +866,10 @@ int launch_int64(wf_ctx *ctx, const wf_plans *plans, const wf_eval_out *out, con
     const wf_dev_problem &dp = ctx->dp;
     uint8_t *scratch = (uint8_t *)ctx->eval_scratch;
     const int64_t units = std::min<int64_t>(ctx->eval_threads, plans->P);
-    if (dp.batch > 0) {
+    if (dp.batch > 0 || (!list && !dp.phi_life && thread_per_plan(dp, ctx->sms, plans->P, true))) {
         const int64_t blocks = (units + kEvalThreads - 1) / kEvalThreads;
-        eval_batched_kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes,
-                                                                      units, list, count);
+        const auto kernel = dp.batch > 0 ? eval_thread_kernel<true> : eval_thread_kernel<false>;
+        kernel<<<(unsigned)blocks, kEvalThreads, 0, st>>>(dp, *plans, *out, scratch, ctx->eval_row_bytes, units, list, count);
     } else {
         const size_t bytes = warp_bytes<uint64_t>(dp, kSolo);
         // A list is most often empty: few CTAs where that can be.
@@ -1123,6 +1143,31 @@ eval_static_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *s, 
     put_result(dp, out, p, st, r, *(const int64_t *)s);
 }
 
+// The same with a thread per plan (thread_per_plan), in the plan's scratch row.
+__global__ void __launch_bounds__(kEvalThreads)
+eval_static_thread_kernel(wf_dev_problem dp, wf_plans pl, wf_eval_out out, uint8_t *s, StaticLayout l, size_t row_bytes)
+{
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= pl.P) return;
+    uint32_t st = WF_ST_TABLES;
+    int64_t mk = WF_INF64, p95 = WF_INF64, g = WF_INF64;
+    if ((*(volatile int *)(s + 8) & 0xFF) != kStaticBadTables) {  // (else nothing is evaluated)
+        wf_dev_problem d = dp;
+        d.first_arrival = *(const int64_t *)s;
+        Row row = row_at(d, s + l.rows + (size_t)p * row_bytes);
+        const PlanRows pr = plan_rows(pl, p);
+        st = plan_status(d, pr, row);
+        if (!st) {
+            play<false>(d, pr, row, 0, &mk, &g);
+            p95 = select_rank(row.comp, d.W, p95_rank(d.W));
+        }
+    }
+    out.status[p] = st;
+    out.makespan_us[p] = mk;
+    out.p95_us[p] = p95;
+    out.gpu_us[p] = g;
+}
+
 // Device address of the static array per device, from the last lookup
 // outside stream capture.
 uint8_t *g_static_addr[64];
@@ -1218,6 +1263,11 @@ extern "C" int wf_eval_plans_static(const wf_problem *pb, const wf_plans *pl, co
     int sms = 0;
     rc = wf_cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
     if (rc) return rc;
+    if (thread_per_plan(dp, sms, pl->P, false)) {
+        eval_static_thread_kernel<<<(unsigned)((pl->P + kEvalThreads - 1) / kEvalThreads), kEvalThreads, 0, st>>>(
+            dp, *pl, *out, s, l, row);
+        return wf_cuda_check(cudaGetLastError(), "static evaluation launch");
+    }
     const WarpShape shape = warp_shape(sms, pl->P, warp_bytes<uint32_t>(dp, kSolo), kSolo32);
     const size_t smem = warps_of(shape) * warp_bytes<uint32_t>(dp, shape);
     const auto by_shape = [&](auto q) {

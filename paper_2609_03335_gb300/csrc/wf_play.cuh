@@ -152,7 +152,8 @@ __device__ __forceinline__ uint2 settle_lru(Q &q, uint32_t &n, uint32_t &u_d, ui
 // then its first entries, and the model goes back in last.  The first three
 // victims' weights are read at once and taken without branching (a loop over
 // victims waited for one weight at a time: about 130 instructions a unit with
-// it, half of that without); weight holds 16 entries, 0 beyond the models.
+// it, half of that without); kRare: where few lanes settle at once and a unit
+// seldom evicts, that is skipped.  weight holds 16 entries, 0 beyond the models.
 // Returns the record's rewritten (w1, w3): the
 // load the unit waits for (none on a hit, Eq. 5) and the occupancy changes.
 template <typename Q>
@@ -184,6 +185,7 @@ struct DevState<uint32_t> {
     uint2 v;  // queue, free capacity
     __device__ __forceinline__ void init(uint32_t cap) { v = make_uint2(~0u, cap); }
     __device__ __forceinline__ bool occupied() const { return v.x != ~0u; }
+    template <bool kRare = false>
     __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
                                             int32_t D, int *err, bool &missed)
     {
@@ -197,7 +199,8 @@ struct DevState<uint32_t> {
         const uint32_t below = ((z & (0u - z)) >> 3) - 1u;  // the bits below that nibble (all when there is none)
         q = (q & below) | ((q >> 4) & ~below) | 0xF0000000u;
         const uint32_t need = hit ? r1 : wm + r1;  // at most the capacity
-        const int e4 = evict(q, need, f, 32, weight);
+        int e4 = 0;
+        if (!kRare || need > f) e4 = evict(q, need, f, 32, weight);
         if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
         q = __funnelshift_rc(q, ~0u, e4);
         const uint32_t gap = q & 0x88888888u;
@@ -221,6 +224,7 @@ struct DevState<uint64_t> {
     uint4 v;  // queue (low, high), free capacity, models held
     __device__ __forceinline__ void init(uint32_t cap) { v = make_uint4(~0u, ~0u, cap, 0u); }
     __device__ __forceinline__ bool occupied() const { return v.w != 0; }
+    template <bool kRare = false>
     __device__ __forceinline__ uint2 settle(uint32_t r1, uint32_t r3, const int32_t *weight, const int32_t *load,
                                             int32_t D, int *err, bool &missed)
     {
@@ -238,7 +242,8 @@ struct DevState<uint64_t> {
         q = (q & below) | ((q >> 4) & ~below) | (hit ? 0xFull << 60 : 0ull);
         n -= hit ? 1u : 0u;
         const uint32_t need = hit ? r1 : wm + r1;
-        const int e4 = evict(q, need, f, (int)(4 * n), weight);
+        int e4 = 0;
+        if (!kRare || need > f) e4 = evict(q, need, f, (int)(4 * n), weight);
         if (need > f) atomicExch(err, 2);  // unreachable for a valid plan
         q = e4 < 64 ? (q >> e4) | ~(~0ull >> e4) : ~0ull;
         n -= (uint32_t)e4 >> 2;

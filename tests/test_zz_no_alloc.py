@@ -190,6 +190,44 @@ def test_large_batches_of_short_windows(D, M, scale):
             assert np.array_equal(a, b[:P])
 
 
+@pytest.mark.parametrize("D,n,M,scale", [(1, 60, 1, 1), (2, 60, 5, 1), (2, 61, 5, 1), (3, 40, 9, 1), (4, 30, 3, 1), (4, 40, 3, 1), (4, 41, 3, 1),
+                                         (4, 12, 4, 1 << 20)])
+def test_large_batches_on_few_devices(D, n, M, scale):
+    """Batches around the one from which short windows on up to four devices
+    take a thread per plan (160 plans an SM), the longest such window and the
+    next, in the static call and on the int64 path; retain rows, invalid plans,
+    run times that leave 32 bits; and tables that fail the device check."""
+    import torch
+    from gpu_util import assert_same, gpu_eval
+    from randprob import random_problem
+    from paper_2609_03335_gb300 import build, wf
+    build.build()
+    most = 160 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(70 + n)
+    prob = random_problem(rng, n_sessions=2, sizes=(n // 2, n - n // 2), D=D, M=M)
+    while prob.N != n:
+        prob = random_problem(rng, n_sessions=2, sizes=(n // 2, n - n // 2), D=D, M=M)
+    prob = prob.with_(lat_us=np.minimum(prob.lat_us.astype(np.int64) * scale, 2**31 - 1).astype(np.int32))
+    plans = wfgen.make_plans(prob, most + 1, 5, p_retain=0.7 if D % 2 else None)
+    plans.place[2, 0] = prob.D
+    plans.order[4, 0] = plans.order[4, 1]
+    want = oracle.eval_plans(prob, plans, threads=8)
+    dprob = wf.DeviceProblem(prob)
+    for P in (most + 1, most):
+        sub = plans.slice(0, P)
+        out = wf.Results(P)
+        wf.wf_eval_plans_static(dprob, wf.DevicePlans.from_host(sub, "cuda"), out)
+        wf.wf_static_status()
+        for a, b in zip(out.numpy(), want):
+            assert np.array_equal(a, b[:P])
+        assert_same(gpu_eval(prob, sub, int64_path=True), dict(zip(("makespan", "p95", "gpu", "status"), (w[:P] for w in want))))
+    dprob.tensors["model"][n - 1] = M
+    wf.wf_eval_plans_static(dprob, wf.DevicePlans.from_host(plans, "cuda"), out := wf.Results(most + 1))
+    with pytest.raises(wf.WfError):
+        wf.wf_static_status()
+    assert (out.numpy()[3] == wf.ST_TABLES).all() and (out.numpy()[0] == wf.INT64_MAX).all()
+
+
 @pytest.mark.parametrize("others", [[1] * 19, [1] * 3 + [0] * 16, [0] * 19, [3, 2, 1, 1, 0, 0], [1] * 250 + [2] * 60 + [0] * 5,
                                     [1] * 900 + [0] * 200])
 def test_static_entry_with_sessions_that_own_no_activation(others):
