@@ -1406,11 +1406,23 @@ int launch_pc_q(const wf_ctx *ctx, int kp, int resident, const wf_plans *pl, con
 // 198 and 198, 487 and 465, but N = 64 in three 209 and 244, 505 and 571; M = 5,
 // D = 3, N = 80 in two 480 and 462.  Up to four models four
 // lanes a plan win from N = 24 on, and lose 2 % below.
-static bool lane_per_plan(const wf_ctx *ctx, int64_t P)
+//
+// Beyond eight models lanes per model have registers for three CTAs an SM, a
+// lane per plan for four: a batch that fills a fourth of each SM and no more
+// is one wave instead of two.  8,500 plans of D = 8, M = 12, N = 163, 400, 1,000:
+// 268, 593, 1,445 and 233, 541, 1,274; N = 2,000, of which shared memory holds three CTAs,
+// 2,825 and 4,508.
+// Returns the shared memory of such a CTA, 0 for a lane per model.
+static size_t lane_per_plan(const wf_ctx *ctx, int64_t P)
 {
     const wf_dev_problem &dp = ctx->dp;
-    if (!dp.reclaim || dp.M <= 4 || P <= 40 * (int64_t)ctx->sms) return false;
-    return dp.N <= (dp.M > 8 ? 32 + 8 * dp.D : dp.N >= 32 * dp.W ? 96 : 24 + 2 * dp.D);
+    if (!dp.reclaim || dp.M <= 4 || P <= 40 * (int64_t)ctx->sms) return 0;
+    const size_t smem = dp.phi_life ? pc_layout<kPlans32, uint32_t, kNuPlan, true>(dp.D, dp.M, dp.W, dp.nslots + 2).total
+                                    : pc_layout<kPlans32, uint32_t, kNuPlan, false>(dp.D, dp.M, dp.W, dp.nslots + 2).total;
+    const bool four = 4 * (smem + 1024) <= 228 * 1024;  // CTAs an SM
+    const int64_t ctas = (P + kPlans32 - 1) / kPlans32;
+    if (dp.M > 8 && four && ctas > 3 * (int64_t)ctx->sms && ctas <= 4 * (int64_t)ctx->sms) return smem;
+    return dp.N <= (dp.M > 8 ? 32 + 8 * dp.D : dp.N >= 32 * dp.W ? 96 : 24 + 2 * dp.D) ? smem : 0;
 }
 
 int wf_launch_nextuse(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, cudaStream_t st)
@@ -1565,15 +1577,12 @@ int wf_launch_sweep(wf_ctx *ctx, const wf_plans *pl, const wf_eval_out *out, con
         // u32 times for every plan; the plans that leave 32 bits go on to the
         // u64 sweep, and from there (or straight) to the int64 path.
         const wf_dev_problem &dp = ctx->dp;
-        const bool by_plan = lane_per_plan(ctx, pl->P);
-        const size_t smem = !by_plan      ? cfg.smem32
-                            : dp.phi_life ? pc_layout<kPlans32, uint32_t, kNuPlan, true>(dp.D, dp.M, dp.W, dp.nslots + 2).total
-                                          : pc_layout<kPlans32, uint32_t, kNuPlan, false>(dp.D, dp.M, dp.W, dp.nslots + 2).total;
+        const size_t by_plan = lane_per_plan(ctx, pl->P);
         if (by_plan)
-            rc = dp.phi_life ? launch_pc_r<uint32_t, kNuPlan, true>(ctx, kPlans32, 1, pl, out, smem, nullptr, nullptr, list1, counts, st)
-                             : launch_pc_r<uint32_t, kNuPlan, false>(ctx, kPlans32, 1, pl, out, smem, nullptr, nullptr, list1, counts, st);
+            rc = dp.phi_life ? launch_pc_r<uint32_t, kNuPlan, true>(ctx, kPlans32, 1, pl, out, by_plan, nullptr, nullptr, list1, counts, st)
+                             : launch_pc_r<uint32_t, kNuPlan, false>(ctx, kPlans32, 1, pl, out, by_plan, nullptr, nullptr, list1, counts, st);
         else
-            rc = launch_pc_q<uint32_t>(ctx, kPlans32, cfg.res32, pl, out, smem, nullptr, nullptr, list1, counts, st);
+            rc = launch_pc_q<uint32_t>(ctx, kPlans32, cfg.res32, pl, out, cfg.smem32, nullptr, nullptr, list1, counts, st);
         if (rc) return rc;
         if (!cfg.smem64) { *rest_list = list1; *rest_count = counts; return WF_OK; }
         rc = launch_pc_q<uint64_t>(ctx, cfg.plans64, cfg.res64, pl, out, cfg.smem64, list1, counts, list2, counts + 1, st);

@@ -171,6 +171,22 @@ def test_long_sessions_in_large_batches(n, sessions):
     assert_same(gpu_eval(prob, plans), oracle_eval(prob, plans))
 
 
+@pytest.mark.parametrize("M", [8, 9, 16])
+def test_batches_of_one_wave_of_four_ctas(M):
+    """Beyond eight models, batches between three and four CTAs an SM take a lane
+    per plan on longer windows too: both ends of that range and one plan beyond
+    each."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(3800 + M)
+    prob = random_problem(rng, n_sessions=20, sizes=(6, 12), D=4, M=M).with_(reclaim=1)
+    assert prob.N > 32 + 8 * 4
+    plans = wfgen.make_plans(prob, 64 * sms + 1, 3, p_retain=0.8)
+    want = oracle_eval(prob, plans)
+    for P in (48 * sms, 48 * sms + 1, 64 * sms, 64 * sms + 1):
+        assert_same(gpu_eval(prob, plans.slice(0, P)), {x: want[x][:P] for x in ("status", "makespan", "p95", "gpu")})
+
+
 def lone_sessions(W, D, M, seed):
     """W sessions of one activation each: as many finish slots as sessions."""
     rng = np.random.default_rng(seed)
